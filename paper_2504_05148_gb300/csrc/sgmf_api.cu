@@ -574,8 +574,13 @@ extern "C" sgmf_status sgmf_compute_batch(sgmf_ctx *c, int n, const uint8_t *lef
       TIMED(c, "agg_sweep", s, launch_agg_sweep(ka, c->b, n, s));
     else
       TIMED(c, "agg_lines", s, launch_agg_lines(ka, c->b, n, c->spill8, s));
-    TIMED(c, "agg_rows_wta", s, launch_agg_rows(ka, c->b, n, c->spill8, s));
-    TIMED(c, "consistency", s, launch_consistency(k, c->b, n, out, s));
+    if (!ka.sweep && c->spill8) {
+      // the line kernels walked the rows too: what is left needs no walk
+      TIMED(c, "agg_rows_wta", s, launch_agg_wta(ka, c->b, n, out, s));
+    } else {
+      TIMED(c, "agg_rows_wta", s, launch_agg_rows(ka, c->b, n, c->spill8, s));
+      TIMED(c, "consistency", s, launch_consistency(k, c->b, n, out, s));
+    }
   }
   c->computed = true;
   c->last_n = n;
@@ -731,16 +736,25 @@ extern "C" sgmf_status sgmf_debug_stage(sgmf_ctx *c, int stage, void *dst, size_
       break;
     }
     case SGMF_STAGE_COST:
-      CUDA_TRY(c, cudaMemcpy2D(dst, need / n, c->b.cost, k.Dp, need / n, n, cudaMemcpyDeviceToHost));
-      break;
-    case SGMF_STAGE_SUM:
+    case SGMF_STAGE_SUM: {
+      const bool u16 = stage == SGMF_STAGE_SUM;
+      const void *src = u16 ? static_cast<const void *>(c->b.dbg_sum) : c->b.cost;
       if (k.band) {   // banded: [H][W][band], cell j = disparity lo_p + j
-        CUDA_TRY(c, cudaMemcpy(dst, c->b.dbg_sum, need, cudaMemcpyDeviceToHost));
+        CUDA_TRY(c, cudaMemcpy(dst, src, need, cudaMemcpyDeviceToHost));
         break;
       }
-      CUDA_TRY(c, cudaMemcpy2D(dst, (size_t)k.D * 2, c->b.dbg_sum, (size_t)k.Dp * 2, (size_t)k.D * 2, n,
-                               cudaMemcpyDeviceToHost));
+      // full range: Dp cells a pixel in group-lane order
+      const size_t es = u16 ? 2 : 1;
+      std::vector<uint8_t> tmp(n * k.Dp * es);
+      CUDA_TRY(c, cudaMemcpy(tmp.data(), src, tmp.size(), cudaMemcpyDeviceToHost));
+      std::vector<int> cell(k.Dp);
+      for (int m = 0; m < k.Dp; ++m) cell[m] = lane_order_cell(k.Dp, u16, m);
+      for (size_t p = 0; p < n; ++p)
+        for (int m = 0; m < k.Dp; ++m)
+          if (cell[m] < k.D)
+            memcpy(static_cast<uint8_t *>(dst) + (p * k.D + cell[m]) * es, &tmp[(p * k.Dp + m) * es], es);
       break;
+    }
   }
   return SGMF_OK;
 }

@@ -1083,20 +1083,10 @@ static cudaError_t launch_line_family_w(const LineArgs &a, int nf, cudaStream_t 
   return cudaGetLastError();
 }
 
-// warps per CTA from the context's tuning (1, 2, 4 or 8); the banded variant
-// exists for 4 warps and up to 8 cells per lane (bands of 64 or 128)
+// four warps a CTA
 template <int CPL, bool S8, int FAM>
 static cudaError_t launch_line_family(const LineArgs &a, int nf, cudaStream_t s) {
-  if (a.lo != nullptr) {
-    if constexpr (CPL <= 8) return launch_line_family_w<CPL, S8, FAM, 4, true>(a, nf, s);
-    return cudaErrorInvalidValue;
-  }
-  switch (a.k.line_warps) {
-    case 1: return launch_line_family_w<CPL, S8, FAM, 1, false>(a, nf, s);
-    case 2: return launch_line_family_w<CPL, S8, FAM, 2, false>(a, nf, s);
-    case 8: return launch_line_family_w<CPL, S8, FAM, 8, false>(a, nf, s);
-    default: return launch_line_family_w<CPL, S8, FAM, 4, false>(a, nf, s);
-  }
+  return launch_line_family_w<CPL, S8, FAM, 4, true>(a, nf, s);
 }
 
 // In banded mode (k.band != 0) the kernels see D = Dp = band: lane cells are
@@ -1161,27 +1151,16 @@ cudaError_t launch_rows_t(const KParams &k, const Buffers &b, int nf, cudaStream
   a.tw = k.tw;
   a.th = k.th;
   a.gate = b.gate;
-  if (k.band) {
-    if constexpr (CPL <= 8) {
-      if (k.sweep) return launch_rows_v<CPL, S8, 2, true, true>(a, nf, s);
-      if (k.num_paths == 8) return launch_rows_v<CPL, S8, 3, true, true>(a, nf, s);
-      return launch_rows_v<CPL, S8, 1, true, true>(a, nf, s);
-    }
-    return cudaErrorInvalidValue;
-  }
-  const bool fulld = k.D == k.Dp;
-  if (k.sweep)
-    return fulld ? launch_rows_v<CPL, S8, 2, true, false>(a, nf, s) : launch_rows_v<CPL, S8, 2, false, false>(a, nf, s);
-  if (k.num_paths == 8)
-    return fulld ? launch_rows_v<CPL, S8, 3, true, false>(a, nf, s) : launch_rows_v<CPL, S8, 3, false, false>(a, nf, s);
-  return fulld ? launch_rows_v<CPL, S8, 1, true, false>(a, nf, s) : launch_rows_v<CPL, S8, 1, false, false>(a, nf, s);
+  if (k.sweep) return launch_rows_v<CPL, S8, 2, true, true>(a, nf, s);
+  if (k.num_paths == 8) return launch_rows_v<CPL, S8, 3, true, true>(a, nf, s);
+  return launch_rows_v<CPL, S8, 1, true, true>(a, nf, s);
 }
 
 }  // namespace sgmf
 
 // explicit instantiations of one lane width (CPL cells per lane); the
-// instantiating file includes sgmf_sweep.cuh
-#define SGMF_AGG_INSTANTIATE(CPL)                                                                        \
+// instantiating file includes sgmf_band_sweep.cuh
+#define SGMF_BAND_INSTANTIATE(CPL)                                                                        \
   namespace sgmf {                                                                                      \
   template cudaError_t launch_lines_t<CPL, false>(const KParams &, const Buffers &, int, cudaStream_t); \
   template cudaError_t launch_lines_t<CPL, true>(const KParams &, const Buffers &, int, cudaStream_t);  \

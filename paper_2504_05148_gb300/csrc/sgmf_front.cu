@@ -649,13 +649,11 @@ __global__ void __launch_bounds__(256) k_cost_seg(KParams k, Buffers b0, const _
   __syncthreads();
   // (2) the cost bytes, four pixels per warp at a time
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-  uint8_t *out = b.cost + (rowp + x0) * Dp + DPL * lane;
+  uint8_t *out = b.cost + (rowp + x0) * Dp;
   for (int xb = P * warp; xb < npx; xb += P * nwarp) {
     uint32_t o[P][DPL];
     cost_quad<CT, DPL>(cr_s, cl_s, pd_s, xb, x0 + xb, lane, k.D, k.nbits, tab_s, o);
-#pragma unroll
-    for (int u = 0; u < P; ++u)
-      if (xb + u < npx) store_cost_bytes<DPL>(out + (size_t)(xb + u) * Dp, o[u]);
+    store_cost_quad<DPL>(out + (size_t)xb * Dp, o, lane, npx - xb);
   }
 }
 

@@ -6,7 +6,8 @@
 //   census          u32 (CS 9x7) or u64 (9x7) [F][H][W]
 //   box-OR masks    u32    [F][MW][H][W]   bit d of word-plane d/32 set when a
 //                                           sparse disparity of the window is d
-//   cost C-bar      uint8  [F][H][W][Dp]   Dp = 32 * DPL >= D, cells d >= D hold 0
+//   cost C-bar      uint8  [F][H][W][Dp]   Dp = 32 * DPL >= D, cells d >= D hold 0;
+//                                           full range: cells in group-lane order (sgmf_lanes.cuh)
 //   partial sums    u16    [F][H][W][Dp]   one per line family (vertical, two diagonals)
 //   spills          uint8/u16 [F][4][line][pos][Dp]  first-direction path costs of a line
 // F is the number of frames a context holds (its batch capacity); every
@@ -146,6 +147,90 @@ __device__ __forceinline__ void store_cost_bytes(uint8_t *o, const uint32_t (&b)
   }
 }
 
+// Four pixels' bytes into the full-range volume, whose cells lie in the order of
+// the aggregation kernels' lanes (sgmf_lanes.cuh): with CPL = 4 DPL cells a
+// group lane, cell w of a group lane and cell w + CPL / 2 are neighbours.  The
+// cost kernel's lanes 4 j .. 4 j + 3 hold group lane j's cells; lanes s and s + 2
+// of them hold the two halves of the same pairs: the first takes both halves
+// of pixels 0 and 1, the second those of pixels 2 and 3, so that every word
+// they exchange is used.  out: the first pixel's Dp bytes; n: its pixels inside
+// the row segment.  Called by the whole warp.
+template <int DPL>
+__device__ __forceinline__ void store_cost_quad(uint8_t *out, const uint32_t (&b)[4][DPL], int lane, int n) {
+  constexpr int Dp = 32 * DPL;
+  const int j = lane >> 2, h = lane & 1;       // group lane, half of its pairs
+  const bool a = (lane & 2) == 0;              // holds the low cells of its pairs
+  auto pack4 = [](uint32_t x0, uint32_t x1, uint32_t x2, uint32_t x3) {
+    return prmt(prmt(x0, x1, 0x1140), prmt(x2, x3, 0x1140), 0x5410);
+  };
+  auto swap = [](uint32_t v) { return __shfl_xor_sync(0xffffffffu, v, 2); };
+  // (own, partner's) -> pairs of bytes (low cell, high cell), first and second two
+  const uint32_t s0 = a ? 0x5140u : 0x1504u, s1 = a ? 0x7362u : 0x3726u;
+  const int u0 = a ? 0 : 2;                    // the lane's first pixel
+  uint8_t *o0 = out + (size_t)u0 * Dp, *o1 = o0 + Dp;
+  if constexpr (DPL == 2) {
+    const uint32_t w01 = pack4(b[0][0], b[0][1], b[1][0], b[1][1]), w23 = pack4(b[2][0], b[2][1], b[3][0], b[3][1]);
+    const uint32_t own = a ? w01 : w23, oth = swap(a ? w23 : w01);
+    if (u0 < n) *reinterpret_cast<uint32_t *>(o0 + j * 8 + h * 4) = prmt(own, oth, s0);
+    if (u0 + 1 < n) *reinterpret_cast<uint32_t *>(o1 + j * 8 + h * 4) = prmt(own, oth, s1);
+  } else if constexpr (DPL == 4) {
+    uint32_t w[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) w[u] = pack4(b[u][0], b[u][1], b[u][2], b[u][3]);
+    const uint32_t k0 = a ? w[0] : w[2], k1 = a ? w[1] : w[3];
+    const uint32_t r0 = swap(a ? w[2] : w[0]), r1 = swap(a ? w[3] : w[1]);
+    if (u0 < n) *reinterpret_cast<uint2 *>(o0 + j * 16 + h * 8) = make_uint2(prmt(k0, r0, s0), prmt(k0, r0, s1));
+    if (u0 + 1 < n) *reinterpret_cast<uint2 *>(o1 + j * 16 + h * 8) = make_uint2(prmt(k1, r1, s0), prmt(k1, r1, s1));
+  } else if constexpr (DPL == 6) {
+    uint32_t w[4], v[2];                       // cells 0 .. 3 of each pixel; cells 4, 5 of two pixels
+#pragma unroll
+    for (int u = 0; u < 4; ++u) w[u] = pack4(b[u][0], b[u][1], b[u][2], b[u][3]);
+    v[0] = pack4(b[0][4], b[0][5], b[1][4], b[1][5]);
+    v[1] = pack4(b[2][4], b[2][5], b[3][4], b[3][5]);
+    const uint32_t k0 = a ? w[0] : w[2], k1 = a ? w[1] : w[3], kv = a ? v[0] : v[1];
+    const uint32_t r0 = swap(a ? w[2] : w[0]), r1 = swap(a ? w[3] : w[1]), rv = swap(a ? v[1] : v[0]);
+    uint32_t *q0 = reinterpret_cast<uint32_t *>(o0 + j * 24 + h * 12), *q1 = reinterpret_cast<uint32_t *>(o1 + j * 24 + h * 12);
+    if (u0 < n) q0[0] = prmt(k0, r0, s0), q0[1] = prmt(k0, r0, s1), q0[2] = prmt(kv, rv, s0);
+    if (u0 + 1 < n) q1[0] = prmt(k1, r1, s0), q1[1] = prmt(k1, r1, s1), q1[2] = prmt(kv, rv, s1);
+  } else {
+    uint32_t w[4][2];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      w[u][0] = pack4(b[u][0], b[u][1], b[u][2], b[u][3]);
+      w[u][1] = pack4(b[u][4], b[u][5], b[u][6], b[u][7]);
+    }
+    uint32_t k[2][2], r[2][2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        k[u][q] = a ? w[u][q] : w[u + 2][q];
+        r[u][q] = swap(a ? w[u + 2][q] : w[u][q]);
+      }
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+      if (u0 + u < n)
+        *reinterpret_cast<uint4 *>((u ? o1 : o0) + h * 128 + j * 16) =
+            make_uint4(prmt(k[u][0], r[u][0], s0), prmt(k[u][0], r[u][0], s1), prmt(k[u][1], r[u][1], s0),
+                       prmt(k[u][1], r[u][1], s1));
+  }
+}
+
+// cell of the group-lane order's position m in the byte form (u16 = false) or
+// the u16 form of a full-range vector of Dp cells (host: debug copies)
+inline int lane_order_cell(int Dp, bool u16, int m) {
+  const int CPL = Dp / 8, NW = CPL / 2;
+  int j, b;
+  if (u16 ? (CPL == 16 || CPL == 32) : CPL == 32) {   // interleaved 16-byte chunks
+    const int per = u16 ? 8 : 16;                     // cells of a chunk
+    j = m % (8 * per) / per;
+    b = m / (8 * per) * per + m % per;
+  } else {
+    j = m / CPL;
+    b = m % CPL;
+  }
+  return j * CPL + (b >> 1) + (b & 1) * NW;
+}
 
 // sticky error word: first error wins
 __device__ __forceinline__ void set_error(int *err, int code) {
@@ -288,6 +373,8 @@ cudaError_t launch_semidense(const KParams &k, const Buffers &b, int nf, cudaStr
 cudaError_t launch_cost(const KParams &k, const Buffers &b, int nf, cudaStream_t s);
 cudaError_t launch_agg_lines(const KParams &k, const Buffers &b, int nf, bool spill8, cudaStream_t s);
 cudaError_t launch_agg_rows(const KParams &k, const Buffers &b, int nf, bool spill8, cudaStream_t s);
+// S, d*, d' and the check from the line walks' byte vectors (rows among them)
+cudaError_t launch_agg_wta(const KParams &k, const Buffers &b, int nf, int16_t *out, cudaStream_t s);
 // the six vertical/diagonal directions as two cluster sweeps (k.sweep, clusters of
 // k.sweep_cs CTAs); plan: the cluster size for the context's shape and batch capacity nb on
 // this device, 0 if none, and in *slots the number of such clusters the device holds at once

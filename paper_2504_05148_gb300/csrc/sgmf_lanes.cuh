@@ -1,0 +1,311 @@
+// sgmf_lanes.cuh -- the lane layout and the recursion step (Eq. 2) of the
+// full-range aggregation kernels.
+//
+// A group of 8 lanes holds the Dp disparities of one path-cost vector; lane j
+// holds cells [j CPL, (j + 1) CPL), CPL = Dp / 8, as NW = CPL / 2 u16x2 words.
+// Word w pairs the cells w (low half) and w + NW (high half), so the d - 1 and
+// d + 1 neighbours of a word are the words w - 1 and w + 1 themselves: only
+// the first and the last word need a byte permute and a shuffle, where words
+// of adjacent cells need a permute per word.  One step of Eq. 2 on a word:
+//   t     = viaddmin(vimin3(L(d-1), L(d+1), m + P2 - P1), P1, L(d))
+//         = min{ L(d), L(d-1)+P1, L(d+1)+P1, m+P2 }
+//   L'(d) = t + C(d) - m                      (one 32-bit add: t >= m per half)
+// with m = min_k L(k), a per-lane u16x2 min and three shuffles.  A warp steps
+// four vectors at once; a step's fixed work (two neighbour shuffles, the
+// minimum's four, a few words of bookkeeping) serves 4 Dp cells.  The 16-lane
+// groups of adjacent-cell words that this replaced spent two full-warp
+// reductions and Dp / 16 + 1 permutes per 2 Dp cells: at D = 128 a sweep over
+// six directions took 592 instructions per 512 cells, now 445 (1242 x 375, one
+// wave of frames: 786 -> 602 us).  A step and its minimum alone are 42
+// instructions at D = 128, 37 of them on the ALU pipe, 176 cycles from step to
+// step when nothing hides them and about 80 when two or more warps do.
+//
+// A path start is the same step applied to an all-zero previous vector (with
+// m = 0 it yields L = C).  Disparities d >= D are padding: their cost is
+// raised by kInf so they never reach the min.
+//
+// Memory order of a vector.  Bytes: a lane's CPL bytes are the words' (low,
+// high) cells in turn, so one permute turns two words into four bytes and one
+// per word back.  u16: the words as they are.  A lane's bytes are one or more
+// chunks of one vector access (16 bytes, 8 where CPL is no multiple of 16);
+// for CPL = 32 (bytes) and CPL = 16, 32 (u16) the chunks of the 8 lanes are
+// interleaved, chunk 0 of every lane first, so that a group's access covers
+// 128 consecutive bytes of shared or global memory.
+#pragma once
+#include <cstdint>
+
+#include "sgmf_internal.cuh"
+
+namespace sgmf {
+namespace oct {
+
+constexpr unsigned kAll = 0xffffffffu;
+constexpr int kGL = 8;          // lanes per group
+constexpr int kGW = 32 / kGL;   // groups (vectors) per warp
+
+// bytes of one chunk, chunks per lane, and the byte offset of lane lig's first
+// chunk and of the next one, for the u8 and the u16 form of a vector
+template <int CPL>
+struct Vec8 {
+  static constexpr int CH = CPL % 16 == 0 ? 16 : 8, N = CPL / CH;
+  static constexpr int kLane = CPL == 32 ? 16 : CPL, kNext = CPL == 32 ? 128 : CH;
+};
+template <int CPL>
+struct Vec16 {
+  static constexpr int N = CPL / 8;
+  static constexpr bool kInter = CPL == 16 || CPL == 32;
+  static constexpr int kLane = kInter ? 16 : 2 * CPL, kNext = kInter ? 128 : 16;
+};
+
+// the u8 chunks at p (the lane's first chunk) as raw 32-bit words
+template <int CPL>
+struct Raw8 {
+  uint32_t v[CPL / 4];
+};
+
+template <int CPL, bool NC>
+__device__ __forceinline__ void load_raw8(const uint8_t *p, Raw8<CPL> &r) {
+  using V = Vec8<CPL>;
+#pragma unroll
+  for (int q = 0; q < V::N; ++q) {
+    if constexpr (V::CH == 16) {
+      const uint4 *s = reinterpret_cast<const uint4 *>(p + q * V::kNext);
+      const uint4 t = NC ? __ldg(s) : *s;
+      r.v[4 * q] = t.x, r.v[4 * q + 1] = t.y, r.v[4 * q + 2] = t.z, r.v[4 * q + 3] = t.w;
+    } else {
+      const uint2 *s = reinterpret_cast<const uint2 *>(p + q * V::kNext);
+      const uint2 t = NC ? __ldg(s) : *s;
+      r.v[2 * q] = t.x, r.v[2 * q + 1] = t.y;
+    }
+  }
+}
+
+// raw bytes -> words; z holds the pad bytes (0x40 for cells d >= D), which
+// become the high bytes
+template <int CPL>
+__device__ __forceinline__ void expand8(const Raw8<CPL> &r, const uint32_t (&z)[CPL / 4], uint32_t (&w)[CPL / 2]) {
+#pragma unroll
+  for (int j = 0; j < CPL / 4; ++j) {
+    w[2 * j] = prmt(r.v[j], z[j], 0x5140);
+    w[2 * j + 1] = prmt(r.v[j], z[j], 0x7362);
+  }
+}
+
+template <int CPL>
+__device__ __forceinline__ void load_u8(const uint8_t *p, const uint32_t (&z)[CPL / 4], uint32_t (&w)[CPL / 2]) {
+  Raw8<CPL> r;
+  load_raw8<CPL, false>(p, r);
+  expand8<CPL>(r, z, w);
+}
+
+// words -> bytes (every real value is <= 255 when used)
+template <int CPL>
+__device__ __forceinline__ void store_u8(uint8_t *p, const uint32_t (&w)[CPL / 2]) {
+  using V = Vec8<CPL>;
+  uint32_t v[CPL / 4];
+#pragma unroll
+  for (int j = 0; j < CPL / 4; ++j) v[j] = prmt(w[2 * j], w[2 * j + 1], 0x6420);
+#pragma unroll
+  for (int q = 0; q < V::N; ++q) {
+    if constexpr (V::CH == 16)
+      *reinterpret_cast<uint4 *>(p + q * V::kNext) = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    else
+      *reinterpret_cast<uint2 *>(p + q * V::kNext) = make_uint2(v[2 * q], v[2 * q + 1]);
+  }
+}
+
+template <int CPL>
+__device__ __forceinline__ void load_u16(const uint8_t *p, uint32_t (&w)[CPL / 2]) {
+  using V = Vec16<CPL>;
+#pragma unroll
+  for (int q = 0; q < V::N; ++q) {
+    const uint4 t = *reinterpret_cast<const uint4 *>(p + q * V::kNext);
+    w[4 * q] = t.x, w[4 * q + 1] = t.y, w[4 * q + 2] = t.z, w[4 * q + 3] = t.w;
+  }
+}
+
+template <int CPL>
+__device__ __forceinline__ void store_u16(uint8_t *p, const uint32_t (&w)[CPL / 2]) {
+  using V = Vec16<CPL>;
+#pragma unroll
+  for (int q = 0; q < V::N; ++q)
+    *reinterpret_cast<uint4 *>(p + q * V::kNext) = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+}
+
+// a vector in the width its path costs need: bytes (S8) or u16
+template <int CPL, bool S8>
+struct VecW {
+  static constexpr int kLane = S8 ? Vec8<CPL>::kLane : Vec16<CPL>::kLane, SB = S8 ? 1 : 2;
+  static __device__ __forceinline__ void put(uint8_t *p, const uint32_t (&w)[CPL / 2]) {
+    if constexpr (S8)
+      store_u8<CPL>(p, w);
+    else
+      store_u16<CPL>(p, w);
+  }
+  static __device__ __forceinline__ void get(const uint8_t *p, uint32_t (&w)[CPL / 2]) {
+    if constexpr (S8) {
+      const uint32_t z[CPL / 4] = {};
+      load_u8<CPL>(p, z, w);
+    } else {
+      load_u16<CPL>(p, w);
+    }
+  }
+};
+
+// asynchronous copies of a lane's own pieces into shared memory
+template <int B>
+__device__ __forceinline__ void cp_async(uint32_t dst, const uint8_t *src) {
+  if constexpr (B == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// a lane's pieces of a byte / u16 vector: global (lane's first chunk) -> slot,
+// and slot -> registers.  slot: the vector's place in the slot, before the lane offset
+template <int CPL>
+__device__ __forceinline__ void copy8(uint32_t slot, int lane, const uint8_t *src) {
+  using V = Vec8<CPL>;
+#pragma unroll
+  for (int q = 0; q < V::N; ++q) cp_async<V::CH>(slot + (q * 32 + lane) * V::CH, src + q * V::kNext);
+}
+template <int CPL>
+__device__ __forceinline__ void copy16(uint32_t slot, int lane, const uint8_t *src) {
+  using V = Vec16<CPL>;
+#pragma unroll
+  for (int q = 0; q < V::N; ++q) cp_async<16>(slot + (q * 32 + lane) * 16, src + q * V::kNext);
+}
+template <int CPL>
+__device__ __forceinline__ void slot_raw8(const uint8_t *slot, int lane, Raw8<CPL> &r) {
+  using V = Vec8<CPL>;
+#pragma unroll
+  for (int q = 0; q < V::N; ++q) {
+    if constexpr (V::CH == 16) {
+      const uint4 t = reinterpret_cast<const uint4 *>(slot)[q * 32 + lane];
+      r.v[4 * q] = t.x, r.v[4 * q + 1] = t.y, r.v[4 * q + 2] = t.z, r.v[4 * q + 3] = t.w;
+    } else {
+      const uint2 t = reinterpret_cast<const uint2 *>(slot)[q * 32 + lane];
+      r.v[2 * q] = t.x, r.v[2 * q + 1] = t.y;
+    }
+  }
+}
+template <int CPL>
+__device__ __forceinline__ void slot8(const uint8_t *slot, int lane, const uint32_t (&z)[CPL / 4],
+                                      uint32_t (&w)[CPL / 2]) {
+  Raw8<CPL> r;
+  slot_raw8<CPL>(slot, lane, r);
+  expand8<CPL>(r, z, w);
+}
+template <int CPL>
+__device__ __forceinline__ void slot16(const uint8_t *slot, int lane, uint32_t (&w)[CPL / 2]) {
+#pragma unroll
+  for (int q = 0; q < Vec16<CPL>::N; ++q) {
+    const uint4 t = reinterpret_cast<const uint4 *>(slot)[q * 32 + lane];
+    w[4 * q] = t.x, w[4 * q + 1] = t.y, w[4 * q + 2] = t.z, w[4 * q + 3] = t.w;
+  }
+}
+
+// pad bytes of the lane's cells d >= D, in the order of the lane's bytes
+template <int CPL>
+__device__ __forceinline__ void pad_bytes(int D, int lig, uint32_t (&z)[CPL / 4]) {
+#pragma unroll
+  for (int i = 0; i < CPL / 4; ++i) {
+    uint32_t v = 0;
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+      if (lig * CPL + 2 * i + (b >> 1) + (b & 1) * (CPL / 2) >= D) v |= (kInf >> 8) << (8 * b);
+    z[i] = v;
+  }
+}
+
+
+struct StepConsts {
+  uint32_t p1x2;   // P1 in both halves
+  uint32_t dpx2;   // (P2 - P1) in both halves
+};
+
+// One step of Eq. 2 for the lane's words.  mm = min_k L(p - r, k) in both
+// halves.  lo_edge / hi_edge are 0xffff in the missing neighbour's half on the
+// first / last lane of the group (L(-1), L(Dp) only enter a min), else 0.
+template <int NW>
+__device__ __forceinline__ void step(uint32_t (&L)[NW], const uint32_t (&C)[NW], uint32_t mm, const StepConsts &sc,
+                                     uint32_t lo_edge, uint32_t hi_edge) {
+  const uint32_t below = __shfl_up_sync(kAll, L[NW - 1], 1, kGL);
+  const uint32_t above = __shfl_down_sync(kAll, L[0], 1, kGL);
+  // below the first word: (cell CPL - 1 of the lane below, own cell NW - 1);
+  // above the last: (own cell NW, cell 0 of the lane above)
+  uint32_t left = prmt(below, L[NW - 1], 0x5432) | lo_edge;
+  const uint32_t last = prmt(L[0], above, 0x5432) | hi_edge;
+  const uint32_t cap = mm + sc.dpx2;           // m + P2 - P1 per half
+  const uint32_t negmm = 0u - mm;
+#pragma unroll
+  for (int i = 0; i < NW; ++i) {
+    const uint32_t right = i == NW - 1 ? last : L[i + 1];
+    const uint32_t t = __viaddmin_u16x2(__vimin3_u16x2(left, right, cap), sc.p1x2, L[i]);
+    left = L[i];
+    L[i] = t + C[i] + negmm;
+  }
+}
+
+// min of the lane's words, per half
+template <int NW>
+__device__ __forceinline__ uint32_t lane_min(const uint32_t (&L)[NW]) {
+  if constexpr (NW == 4) {
+    return __vminu2(__vimin3_u16x2(L[0], L[1], L[2]), L[3]);
+  } else if constexpr (NW == 8) {
+    return __vimin3_u16x2(__vimin3_u16x2(L[0], L[1], L[2]), __vimin3_u16x2(L[3], L[4], L[5]), __vminu2(L[6], L[7]));
+  } else {
+    uint32_t v = L[0];
+#pragma unroll
+    for (int i = 1; i + 1 < NW; i += 2) v = __vimin3_u16x2(v, L[i], L[i + 1]);
+    return NW % 2 == 0 ? __vminu2(v, L[NW - 1]) : v;
+  }
+}
+
+// min over the group's disparities, in both halves
+template <int NW>
+__device__ __forceinline__ uint32_t group_min(const uint32_t (&L)[NW]) {
+  uint32_t v = lane_min<NW>(L);
+  v = __vminu2(v, prmt(v, v, 0x1032));
+  // two rounds of shuffles instead of three: they are the step's longest chain
+  const uint32_t a = __shfl_xor_sync(kAll, v, 1), b = __shfl_xor_sync(kAll, v, 2), c = __shfl_xor_sync(kAll, v, 3);
+  v = __vminu2(__vimin3_u16x2(v, a, b), c);
+  return __vminu2(v, __shfl_xor_sync(kAll, v, 4));
+}
+
+// min of a u32 over the group
+__device__ __forceinline__ uint32_t group_min_u32(uint32_t v) {
+#pragma unroll
+  for (int s = 1; s < kGL; s *= 2) v = min(v, __shfl_xor_sync(kAll, v, s));
+  return v;
+}
+
+// Sub-pixel disparity in 1/16 px: the vertex of the parabola through sm =
+// S(d*-1), s0 = S(d*), sp = S(d*+1); 16 d* at the ends of the range.  d* is the
+// smallest argmin: den = sm - 2 s0 + sp > 0 and 16 (sm - sp) > -16 den, so the
+// biased numerator is positive: offset = floor((16 (sm - sp) + den) / (2 den)) =
+// that quotient - 8.
+__device__ __forceinline__ int subpixel_disp(int ds, int D, uint32_t sm, uint32_t s0, uint32_t sp) {
+  int v = 16 * ds;
+  if (ds > 0 && ds < D - 1) {
+    const uint32_t den = sm + sp - 2u * s0;
+    v += (int)((16u * sm + 17u * den - 16u * sp) / (2u * den)) - 8;
+  }
+  return v;
+}
+
+// opt in once per device to the kernel's dynamic shared memory
+template <typename Kern>
+static cudaError_t smem_optin(Kern kern, int bytes, bool (&done)[64]) {
+  return once_per_device(done, [&](int) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  });
+}
+
+}  // namespace oct
+}  // namespace sgmf
