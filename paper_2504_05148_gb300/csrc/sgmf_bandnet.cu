@@ -9,16 +9,18 @@
 // pixels and B the weights: M = 128, N = 32, K = 288 = 18 MMAs of K = 16.
 // The data gradient is the same GEMM on the output gradient with the weights
 // rotated by 180 degrees and transposed; the weight gradient is a GEMM over
-// pixels: D[(tap, ci)][co] = sum_p X[p + o_tap][ci] dY[p][co] (M = 288 in three
-// tiles of 128, N = 32, K = 128 pixels per step).
+// pixels: D[(tap, ci)][co] = sum_p X[p + o_tap][ci] dY[p][co].
 //
-// Shared-memory operands use the K-major layout without swizzle: 8 x 8
-// element core matrices of 128 contiguous bytes (8 rows of 16 bytes); the
-// descriptor's leading byte offset is the step between core matrices along
-// K, its stride byte offset the step between 8-row groups.  One thread
-// issues the MMAs; tcgen05.commit arrives on an mbarrier that every thread
-// waits on (bounded), then each warp reads its 32 accumulator rows with
-// tcgen05.ld.
+// Shared-memory operands use the layouts without swizzle: 8 x 8 element core
+// matrices of 128 contiguous bytes (8 rows of 16 bytes).  Staged activations
+// are chunk planes, [8-channel chunk][pixel][8 channels] of 16 bytes a pixel:
+// read with the channels along K (K-major) the plane step is the descriptor's
+// leading and 128 bytes its stride byte offset; read with the pixels along K
+// (MN-major, the weight gradient) 128 bytes is the leading and the plane step
+// the stride byte offset.  Either way a tap's shift by kx pixels is a start
+// address 16 kx bytes on.  One thread issues the MMAs; tcgen05.commit arrives
+// on an mbarrier that every thread waits on (bounded), then each warp reads
+// its 32 accumulator rows with tcgen05.ld.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -48,22 +50,46 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 // generic-proxy shared-memory writes become visible to the tensor core's reads
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// D (tensor memory) (+)= A (smem) * B (smem)^T, BF16 in, FP32 accumulate
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                          uint32_t accumulate) {
+// one lane of a converged warp
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t e;
   asm volatile(
       "{\n"
       ".reg .pred p;\n"
+      "elect.sync _|p, 0xffffffff;\n"
+      "selp.u32 %0, 1, 0, p;\n"
+      "}\n"
+      : "=r"(e));
+  return e;
+}
+// D (tensor memory) (+)= A (smem) * B (smem)^T, BF16 in, FP32 accumulate.  The
+// whole warp runs the code around it (so that descriptors stay warp-uniform),
+// the lane with leader != 0 issues
+__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                          uint32_t accumulate, uint32_t leader) {
+  asm volatile(
+      "{\n"
+      ".reg .pred p, q;\n"
       "setp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
+      "setp.ne.b32 q, %5, 0;\n"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
       "}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(leader)
       : "memory");
 }
-// arrive on the mbarrier once every MMA issued so far by this thread has completed
-__device__ __forceinline__ void umma_commit(uint64_t *bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
+// arrive on the mbarrier once every MMA issued so far by the leader has completed
+__device__ __forceinline__ void umma_commit(uint64_t *bar, uint32_t leader) {
+  asm volatile(
+      "{\n"
+      ".reg .pred q;\n"
+      "setp.ne.b32 q, %1, 0;\n"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
+      "}\n" ::"r"(smem_u32(bar)),
+      "r"(leader)
+      : "memory");
+}
+__device__ __forceinline__ void bn_arrive(uint64_t *bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 // 32 consecutive accumulator columns of this warp's 32 lanes: thread t gets lane (taddr.lane + t)
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
@@ -90,9 +116,27 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo, uint32_t
   return d;
 }
 
-// instruction descriptor of kind::f16: BF16 A and B (both K-major), FP32 D
-constexpr uint32_t idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+// the descriptor of an operand `bytes` further on (a multiple of 16): the
+// address field is the low 14 bits, and shared memory ends below its range
+__device__ __forceinline__ uint64_t sdesc_at(uint64_t d, uint32_t bytes) {
+  return (d & 0xffffffff00000000ull) | ((uint32_t)d + (bytes >> 4));
+}
+
+// instruction descriptor of kind::f16: BF16 A and B (both K-major, or both
+// MN-major), FP32 D
+constexpr uint32_t idesc_bf16(int M, int N, bool mn_major = false) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | (mn_major ? 3u << 15 : 0u) | ((uint32_t)(N >> 3) << 17) |
+         ((uint32_t)(M >> 4) << 24);
+}
+
+// 16-byte asynchronous copy, zero-filled where !in (src stays a valid address)
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool in) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
 constexpr int kBnC = 32;               // channels
@@ -108,6 +152,11 @@ __host__ __device__ __forceinline__ int cm_off(int row, int k, int kc) {
 __device__ __forceinline__ uint16_t f2bf(float f) {
   const __nv_bfloat16 b = __float2bfloat16_rn(f);
   return *reinterpret_cast<const uint16_t *>(&b);
+}
+// two floats -> packed bf16 (round to nearest even), lo in the low half
+__device__ __forceinline__ uint32_t f2bf2(float lo, float hi) {
+  const __nv_bfloat162 b = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t *>(&b);
 }
 __device__ __forceinline__ float bf2f(uint16_t u) { return __uint_as_float((uint32_t)u << 16); }
 
@@ -146,17 +195,68 @@ struct BnConvArgs {
 // bytes further (stride byte offset) and the second chunk one chunk plane
 // further (leading byte offset).  No im2col copy: 18 MMAs read the same
 // ~25 KB of staged input through different descriptor start addresses.
+// Measured at 16 x 94 x 311 pixels: 30 us, 37 before the pieces' addresses were
+// a compare and an immediate each and the results were packed two at a time.
+// (Warps of their own for loads, issue and epilogue on three cp.async stages
+// and two accumulators: 42 us, as only two such CTAs fit a SM instead of four.)
 constexpr int kCvM = 128, kCvPix = kCvM + 2;           // output pixels, staged pixels per row
 constexpr int kCvPlane = kCvPix * 16;                  // bytes of one chunk plane (2080)
 constexpr int kCvX = 3 * 4 * kCvPlane;                 // 24960 bytes of staged input
-constexpr int kCvSmem = kCvX + kBnB + 16;
+constexpr int kCvSmem = kCvX + kBnB + 32 * 4 + 16;
+
+// Position of a tile: its first pixel x0 of row y of image img.
+struct BnTile {
+  int x0, y, img;
+  __device__ __forceinline__ BnTile(long long tile, int tpr, int h) {
+    const long long row = tile / tpr;
+    x0 = (int)(tile - row * tpr) * kCvM;
+    img = (int)(row / h);
+    y = (int)(row - (long long)img * h);
+  }
+  __device__ __forceinline__ void next(int w, int h) {
+    x0 += kCvM;
+    if (x0 >= w) {
+      x0 = 0;
+      if (++y == h) {
+        y = 0;
+        ++img;
+      }
+    }
+  }
+};
+
+// stage rows y - 1, y, y + 1, pixels x0 - 1 .. x0 + 128 of x as chunk planes
+// (zero outside the image), by THREADS threads: a thread keeps its chunk and
+// its pixels of each row, so that a piece is a compare and a copy
+template <int THREADS>
+__device__ __forceinline__ void bn_stage_rows(uint32_t dst, const uint16_t *x, const BnTile &t, int w, int h) {
+  const int j = threadIdx.x & 3, p0 = threadIdx.x >> 2;
+  const uint16_t *row = x + (((long long)t.img * h + t.y - 1) * w + t.x0 - 1) * kBnC;   // staged pixel 0 of row y - 1
+#pragma unroll
+  for (int ky = 0; ky < 3; ++ky) {
+    const bool row_in = (unsigned)(t.y + ky - 1) < (unsigned)h;
+    const uint16_t *src = row + ((long long)ky * w + p0) * kBnC + 8 * j;
+    const uint32_t d = dst + (ky * 4 + j) * kCvPlane + p0 * 16;
+#pragma unroll
+    for (int s = 0; s < kCvM * 4 / THREADS; ++s) {
+      const bool in = row_in && (unsigned)(t.x0 - 1 + p0 + s * (THREADS / 4)) < (unsigned)w;
+      cp_async16(d + s * (THREADS / 4) * 16, in ? src + s * (THREADS / 4) * kBnC : x, in);
+    }
+  }
+  if (threadIdx.x < 24) {                        // the last two pixels of each row
+    const int ky = threadIdx.x >> 3, px = kCvM + ((threadIdx.x >> 2) & 1);
+    const bool in = (unsigned)(t.y + ky - 1) < (unsigned)h && (unsigned)(t.x0 - 1 + px) < (unsigned)w;
+    cp_async16(dst + (ky * 4 + j) * kCvPlane + px * 16, in ? row + ((long long)ky * w + px) * kBnC + 8 * j : x, in);
+  }
+}
 
 __global__ void __launch_bounds__(128) k_bn_conv(const __grid_constant__ BnConvArgs a, int tiles) {
   extern __shared__ __align__(1024) uint8_t sm[];
   uint8_t *Xs = sm;
   uint8_t *Bs = sm + kCvX;
-  uint64_t *bar = reinterpret_cast<uint64_t *>(sm + kCvX + kBnB);
-  uint32_t *slot = reinterpret_cast<uint32_t *>(sm + kCvX + kBnB + 8);
+  float *bias_s = reinterpret_cast<float *>(sm + kCvX + kBnB);
+  uint64_t *bar = reinterpret_cast<uint64_t *>(bias_s + 32);
+  uint32_t *slot = reinterpret_cast<uint32_t *>(bar + 1);
   const int tid = threadIdx.x, warp = tid >> 5;
   if (warp == 0) {
     tmem_alloc(slot, 32);
@@ -166,6 +266,7 @@ __global__ void __launch_bounds__(128) k_bn_conv(const __grid_constant__ BnConvA
     mbar_init(bar, 1);
     mbar_fence_init();
   }
+  if (tid < 32) bias_s[tid] = a.bias ? a.bias[tid] : 0.0f;
   {
     // the packed weights, three loads a thread in flight at a time
     constexpr int kPerThread = kBnB / 16 / 128;
@@ -185,65 +286,68 @@ __global__ void __launch_bounds__(128) k_bn_conv(const __grid_constant__ BnConvA
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *slot;
-  const uint32_t idesc = idesc_bf16(128, 32);
-  // the 16-byte pieces a thread stages: rows y-1, y, y+1, pixels x0-1 ..
-  // x0+128, four chunks each; all of a tile's loads are issued together, and
-  // the next tile's while this one's MMAs and epilogue run
-  constexpr int kPieces = 3 * kCvPix * 4, kPer = (kPieces + 127) / 128;
-  auto fetch = [&](long long tile, uint4 (&v)[kPer]) {
-    const int x0 = (int)(tile % tpr) * kCvM;
-    const long long row = tile / tpr;                        // img * h + y
-    const int y = (int)(row % a.h);
-    const long long img = row / a.h;
+  constexpr uint32_t idesc = idesc_bf16(128, 32);
+  const uint32_t leader = elect_one();
+  // the 16-byte pieces a thread stages (its chunk and its pixels of each of the
+  // three rows, so that a piece is a compare and a load): all of a tile's loads
+  // are issued together, and the next tile's while this one's MMAs and
+  // epilogue run
+  const int j = tid & 3, px0 = tid >> 2;
+  uint4 pf[3][4], pf2;                                       // pixels px0 + 32 s; the rows' last two pixels
+  const int ky2 = tid >> 3, pix2 = kCvM + (px0 & 1);         // (threads 0 .. 23)
+  auto fetch = [&](const BnTile &t) {
+    const uint16_t *row = a.x + (((long long)t.img * a.h + t.y - 1) * a.w + t.x0 - 1) * kBnC + 8 * j;
+    const uint4 zero = make_uint4(0, 0, 0, 0);
 #pragma unroll
-    for (int s = 0; s < kPer; ++s) {
-      const int i = tid + s * 128;
-      const int j = i & 3, px = (i >> 2) % kCvPix, ky = (i >> 2) / kCvPix;
-      const int yy = y + ky - 1, xx = x0 - 1 + px;
-      const bool in = i < kPieces && yy >= 0 && yy < a.h && xx >= 0 && xx < a.w;
-      v[s] = in ? reinterpret_cast<const uint4 *>(a.x + ((img * a.h + yy) * a.w + xx) * kBnC)[j]
-                : make_uint4(0, 0, 0, 0);
+    for (int ky = 0; ky < 3; ++ky) {
+      const bool row_in = (unsigned)(t.y + ky - 1) < (unsigned)a.h;
+      const uint16_t *src = row + ((long long)ky * a.w + px0) * kBnC;
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        pf[ky][s] = zero;
+        if (row_in && (unsigned)(t.x0 - 1 + px0 + 32 * s) < (unsigned)a.w)
+          pf[ky][s] = *reinterpret_cast<const uint4 *>(src + 32 * s * kBnC);
+      }
     }
+    pf2 = zero;
+    if (tid < 24 && (unsigned)(t.y + ky2 - 1) < (unsigned)a.h && (unsigned)(t.x0 - 1 + pix2) < (unsigned)a.w)
+      pf2 = *reinterpret_cast<const uint4 *>(row + ((long long)ky2 * a.w + pix2) * kBnC);
   };
-  uint4 pf[kPer];
   const long long tile0 = (long long)blockIdx.x * tiles;
-  if (tile0 < ntile) fetch(tile0, pf);
+  BnTile cur(tile0, tpr, a.h), nxt = cur;
+  if (tile0 < ntile) fetch(nxt);
   bool ok = true;
   int phase = 0;
   for (int it = 0; it < tiles && ok; ++it) {
     const long long tile = tile0 + it;
     if (tile >= ntile) break;                                // CTA-uniform
-    const int tx = (int)(tile % tpr);
-    const long long row = tile / tpr;                        // img * h + y
-    const int x0 = tx * kCvM;
     // the staged rows as chunk planes
 #pragma unroll
-    for (int s = 0; s < kPer; ++s) {
-      const int i = tid + s * 128;
-      if (i < kPieces) {
-        const int j = i & 3, px = (i >> 2) % kCvPix, ky = (i >> 2) / kCvPix;
-        *reinterpret_cast<uint4 *>(Xs + (ky * 4 + j) * kCvPlane + px * 16) = pf[s];
-      }
-    }
+    for (int ky = 0; ky < 3; ++ky)
+#pragma unroll
+      for (int s = 0; s < 4; ++s)
+        *reinterpret_cast<uint4 *>(Xs + (ky * 4 + j) * kCvPlane + (px0 + 32 * s) * 16) = pf[ky][s];
+    if (tid < 24) *reinterpret_cast<uint4 *>(Xs + (ky2 * 4 + j) * kCvPlane + pix2 * 16) = pf2;
     fence_async_smem();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (tid == 0) {
-      const uint32_t x_0 = smem_u32(Xs), b0 = smem_u32(Bs);
-#pragma unroll 1
+    if (warp == 0) {
+      const uint64_t xd = sdesc(smem_u32(Xs), kCvPlane, 128), bd = sdesc(smem_u32(Bs), 128, kBnKChunks * 128);
+#pragma unroll
       for (int t = 0; t < 9; ++t) {
         const int ky = t / 3, kx = t % 3;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const uint32_t as = x_0 + (ky * 4 + 2 * h) * kCvPlane + kx * 16;
-          umma_bf16(tmem, sdesc(as, kCvPlane, 128), sdesc(b0 + (t * 2 + h) * 256, 128, kBnKChunks * 128), idesc,
-                    (t > 0 || h > 0) ? 1u : 0u);
-        }
+        for (int h = 0; h < 2; ++h)
+          umma_bf16(tmem, sdesc_at(xd, (ky * 4 + 2 * h) * kCvPlane + kx * 16), sdesc_at(bd, (t * 2 + h) * 256), idesc,
+                    (t > 0 || h > 0) ? 1u : 0u, leader);
       }
-      umma_commit(bar);
+      umma_commit(bar, leader);
     }
-    if (it + 1 < tiles && tile + 1 < ntile) fetch(tile + 1, pf);
+    if (it + 1 < tiles && tile + 1 < ntile) {
+      nxt.next(a.w, a.h);
+      fetch(nxt);
+    }
     __syncwarp();
     const bool w_ok = mbar_wait_bounded(bar, (uint32_t)(phase & 1), kWaitLimit);
     ++phase;
@@ -256,12 +360,15 @@ __global__ void __launch_bounds__(128) k_bn_conv(const __grid_constant__ BnConvA
     tc_fence_after();
     float v[32];
     tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16), v);
-    const int x = x0 + tid;
+    const int x = cur.x0 + tid;
     if (x < a.w) {
-      const long long p = row * a.w + x;
+      const long long p = ((long long)cur.img * a.h + cur.y) * a.w + x;
       if (a.bias) {
 #pragma unroll
-        for (int c = 0; c < 32; ++c) v[c] += a.bias[c];
+        for (int c = 0; c < 32; c += 4) {
+          const float4 bv = *reinterpret_cast<const float4 *>(bias_s + c);
+          v[c] += bv.x, v[c + 1] += bv.y, v[c + 2] += bv.z, v[c + 3] += bv.w;
+        }
       }
       if (a.relu) {
 #pragma unroll
@@ -275,10 +382,9 @@ __global__ void __launch_bounds__(128) k_bn_conv(const __grid_constant__ BnConvA
           const uint32_t mw[4] = {m.x, m.y, m.z, m.w};
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            const uint32_t lo = mw[q] & 0xffffu, hi = mw[q] >> 16;
-            // bf16 > 0: sign bit clear and not zero
-            if (!(lo != 0 && !(lo & 0x8000u))) v[8 * j + 2 * q] = 0.0f;
-            if (!(hi != 0 && !(hi & 0x8000u))) v[8 * j + 2 * q + 1] = 0.0f;
+            // bf16 > 0, as a signed 16-bit value: sign bit clear and not zero
+            if ((int16_t)(mw[q] & 0xffffu) <= 0) v[8 * j + 2 * q] = 0.0f;
+            if ((int32_t)mw[q] < 0x10000) v[8 * j + 2 * q + 1] = 0.0f;
           }
         }
       }
@@ -293,12 +399,12 @@ __global__ void __launch_bounds__(128) k_bn_conv(const __grid_constant__ BnConvA
         for (int j = 0; j < 4; ++j) {
           uint32_t u[4];
 #pragma unroll
-          for (int q = 0; q < 4; ++q)
-            u[q] = (uint32_t)f2bf(v[8 * j + 2 * q]) | ((uint32_t)f2bf(v[8 * j + 2 * q + 1]) << 16);
+          for (int q = 0; q < 4; ++q) u[q] = f2bf2(v[8 * j + 2 * q], v[8 * j + 2 * q + 1]);
           o[j] = make_uint4(u[0], u[1], u[2], u[3]);
         }
       }
     }
+    cur.next(a.w, a.h);
     // the accumulator and the staged input are reused by the next tile
     tc_fence_before();
     __syncthreads();
@@ -310,16 +416,26 @@ __global__ void __launch_bounds__(128) k_bn_conv(const __grid_constant__ BnConvA
 }
 
 // ---- weight gradient ---------------------------------------------------------------------
-// Each CTA reduces `chunks` chunks of 128 pixels: per chunk it builds A (3
-// tiles of 128 (tap, ci) rows x 128 pixels; rows 288..383 stay zero) and B
-// (32 co rows x 128 pixels), issues 3 x 8 MMAs into three 32-column
-// accumulators and waits for them before the next chunk.  The accumulators
-// and the bias gradient are written as this CTA's partial sums; a second
-// kernel adds the partials of all CTAs in CTA order, so that the gradient
-// (and with it training) does not depend on the order the CTAs finish in.
-constexpr int kWgA = 128 * 128 * 2;     // one A tile: 32 KiB
-constexpr int kWgB = 32 * 128 * 2;      // 8 KiB
-constexpr int kWgSmem = 3 * kWgA + kWgB + 16;
+// D[(tap, ci)][co] = sum over pixels of X[p + o_tap][ci] dY[p][co].  A CTA
+// reduces `chunks` tiles of 128 pixels of an image row.  X is staged as in the
+// forward pass (three rows, chunk planes) and dY as four chunk planes; with
+// the pixels along K both are MN-major operands as they lie: for a fixed kx
+// the rows (ky, ci) of A are the twelve planes in turn (M = 128 with four
+// planes past them, whose rows are not read back), N = 32 channels of dY, and
+// the tile is eight MMAs of K = 16 pixels into the accumulator of kx.
+// (Transposing both through 2-byte shared-memory stores, 320 a pixel, took
+// 139 us where this takes 47 us: 16 x 94 x 311 pixels; the MMAs' operand reads
+// bound it, about 120 cycles each whatever the number of stages, loading warps
+// and CTAs.)  The accumulators and the bias gradient are written as
+// this CTA's partial sums; a second kernel adds the partials of all CTAs in a
+// fixed order, so that the gradient (and with it training) does not depend on
+// the order the CTAs finish in.
+constexpr int kWgStages = 3, kWgLoad = 8;           // loading warps; one more issues the MMAs
+constexpr int kWgThreads = 32 * kWgLoad;            // loading threads
+constexpr int kWgPlane = kCvM * 16;                 // a chunk plane of dY
+constexpr int kWgStage = 16 * kCvPlane;             // 12 planes of X, then the 4 of dY (and what M = 128 reads past them)
+static_assert(kCvX + 4 * kWgPlane <= kWgStage, "the planes fit the stage");
+constexpr int kWgSmem = kWgStages * kWgStage + 2 * kWgStages * 8 + 16;
 constexpr int kWgMaxCtas = 304;         // about two CTAs per SM
 constexpr int kWgPart = kBnK * 32 + 32; // one CTA's partial: dw [co][tap][ci], then db [co]
 // partial sums of one sgmf_bn_wgrad call (calls must not overlap on the GPU)
@@ -332,136 +448,140 @@ struct BnWgradArgs {
   int *err;
 };
 
-__global__ void __launch_bounds__(128) k_bn_wgrad(const __grid_constant__ BnWgradArgs a) {
+__global__ void __launch_bounds__(kWgThreads + 32) k_bn_wgrad(const __grid_constant__ BnWgradArgs a) {
   extern __shared__ __align__(1024) uint8_t sm[];
-  uint8_t *As = sm;
-  uint8_t *Bs = sm + 3 * kWgA;
-  uint64_t *bar = reinterpret_cast<uint64_t *>(sm + 3 * kWgA + kWgB);
-  uint32_t *slot = reinterpret_cast<uint32_t *>(sm + 3 * kWgA + kWgB + 8);
+  uint64_t *full = reinterpret_cast<uint64_t *>(sm + kWgStages * kWgStage);   // a stage is filled
+  uint64_t *empty = full + kWgStages;                                         // its MMAs are done
+  uint32_t *slot = reinterpret_cast<uint32_t *>(empty + kWgStages);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tpr = (a.w + kCvM - 1) / kCvM;
+  const long long ntile = (long long)a.n * a.h * tpr, tile0 = (long long)blockIdx.x * a.chunks;
+  const int nt = (int)min((long long)a.chunks, ntile - tile0);               // >= 1
   if (warp == 0) {
     tmem_alloc(slot, 128);
     tmem_relinquish();
   }
   if (tid == 0) {
-    mbar_init(bar, 1);
+    for (int s = 0; s < kWgStages; ++s) {
+      mbar_init(&full[s], kWgThreads);
+      mbar_init(&empty[s], 1);
+    }
     mbar_fence_init();
   }
-  // the padding rows 288..383 of the third A tile stay zero
-  for (int i = tid; i < kWgA / 16; i += 128) reinterpret_cast<uint4 *>(As + 2 * kWgA)[i] = make_uint4(0, 0, 0, 0);
-  float dbp[32];
+  // what M = 128 reads past the planes is never used, but starts finite
+  for (int i = tid; i < kWgStages * (kWgStage - kCvX - 4 * kWgPlane) / 16; i += kWgThreads + 32) {
+    constexpr int kTail = (kWgStage - kCvX - 4 * kWgPlane) / 16;
+    reinterpret_cast<uint4 *>(sm + i / kTail * kWgStage + kCvX + 4 * kWgPlane)[i % kTail] = make_uint4(0, 0, 0, 0);
+  }
+  float dbp[8];                                      // bias gradient of the thread's chunk over its pixels
 #pragma unroll
-  for (int c = 0; c < 32; ++c) dbp[c] = 0.0f;
-  const long long P = (long long)a.n * a.h * a.w;
+  for (int c = 0; c < 8; ++c) dbp[c] = 0.0f;
+  fence_async_smem();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *slot;
-  bool ok = true;
-  int issued = 0;
-  for (int ch = 0; ch < a.chunks && ok; ++ch) {
-    const long long p = ((long long)blockIdx.x * a.chunks + ch) * 128 + tid;
-    if ((long long)blockIdx.x * a.chunks * 128 + (long long)ch * 128 >= P) break;   // CTA-uniform
-    const bool live = p < P;
-    int img = 0, py = 0, px = 0;
-    if (live) {
-      img = (int)(p / ((long long)a.h * a.w));
-      const int r = (int)(p % ((long long)a.h * a.w));
-      py = r / a.w;
-      px = r % a.w;
-    }
-    // B: dY of this pixel (column tid), and the bias-gradient partial sums
-    {
-      const uint4 *src = reinterpret_cast<const uint4 *>(a.dy + (live ? p : 0) * kBnC);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const uint4 v = live ? src[j] : make_uint4(0, 0, 0, 0);
-        const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int c0 = 8 * j + 2 * q;
-          *reinterpret_cast<uint16_t *>(Bs + cm_off(c0, tid, 16)) = (uint16_t)(u[q] & 0xffffu);
-          *reinterpret_cast<uint16_t *>(Bs + cm_off(c0 + 1, tid, 16)) = (uint16_t)(u[q] >> 16);
-          dbp[c0] += bf2f((uint16_t)(u[q] & 0xffffu));
-          dbp[c0 + 1] += bf2f((uint16_t)(u[q] >> 16));
-        }
-      }
-    }
-    // A: X at the 9 taps of this pixel (column tid), rows (tap, ci)
-#pragma unroll 1
-    for (int tap = 0; tap < 9; ++tap) {
-      const int yy = py + tap / 3 - 1, xx = px + tap % 3 - 1;
-      const bool in = live && yy >= 0 && yy < a.h && xx >= 0 && xx < a.w;
-      const long long q = in ? ((long long)img * a.h + yy) * a.w + xx : 0;
-      const uint4 *src = reinterpret_cast<const uint4 *>(a.x + q * kBnC);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const uint4 v = in ? src[j] : make_uint4(0, 0, 0, 0);
-        const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int m0 = tap * kBnC + 8 * j + 2 * q;
-          uint8_t *t0 = As + (m0 >> 7) * kWgA, *t1 = As + ((m0 + 1) >> 7) * kWgA;
-          *reinterpret_cast<uint16_t *>(t0 + cm_off(m0 & 127, tid, 16)) = (uint16_t)(u[q] & 0xffffu);
-          *reinterpret_cast<uint16_t *>(t1 + cm_off((m0 + 1) & 127, tid, 16)) = (uint16_t)(u[q] >> 16);
-        }
-      }
-    }
-    fence_async_smem();
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    if (tid == 0) {
-      const uint32_t idesc = idesc_bf16(128, 32);
-      const uint32_t b0 = smem_u32(Bs);
-#pragma unroll 1
-      for (int t = 0; t < 3; ++t) {
-        const uint32_t a0 = smem_u32(As + t * kWgA);
-#pragma unroll 1
-        for (int s = 0; s < 8; ++s)
-          umma_bf16(tmem + 32 * t, sdesc(a0 + s * 256, 128, 16 * 128), sdesc(b0 + s * 256, 128, 16 * 128), idesc,
-                    (ch > 0 || s > 0) ? 1u : 0u);
-      }
-      umma_commit(bar);
-    }
-    __syncwarp();
-    const bool w_ok = mbar_wait_bounded(bar, (uint32_t)(issued & 1), kWaitLimit);
-    ++issued;
-    if (!__syncthreads_and(w_ok)) {
-      if (tid == 0) set_error(a.err, kErrTimeout);
-      mbar_wait_bounded(bar, (uint32_t)((issued - 1) & 1), kWaitLimit);
+  bool ok = true;                                    // this warp's waits
+  auto wait = [&](uint64_t *bar, int use) {
+    const bool w = mbar_wait_bounded(bar, (uint32_t)use & 1u, kWaitLimit);
+    if (!__all_sync(0xffffffffu, w)) {
+      if (lane == 0) set_error(a.err, kErrTimeout);
       ok = false;
     }
-    tc_fence_after();
+    return ok;
+  };
+  if (warp < kWgLoad) {
+    BnTile ld(tile0, tpr, a.h);
+    constexpr int kY = kCvM * 4 / kWgThreads;        // dY pieces a thread stages: its chunk is tid & 3 throughout
+    for (int t = 0; t < nt + kWgStages - 1; ++t) {
+      if (t < nt) {
+        if (t >= kWgStages && !wait(&empty[t % kWgStages], t / kWgStages - 1)) break;
+        const uint32_t dst = smem_u32(sm) + t % kWgStages * kWgStage;
+        bn_stage_rows<kWgThreads>(dst, a.x, ld, a.w, a.h);
+        const uint16_t *src = a.dy + (((long long)ld.img * a.h + ld.y) * a.w + ld.x0) * kBnC + 8 * (tid & 3);
+#pragma unroll
+        for (int s = 0; s < kY; ++s) {
+          const int px = (tid >> 2) + s * (kWgThreads / 4);
+          const bool in = ld.x0 + px < a.w;
+          cp_async16(dst + kCvX + (tid & 3) * kWgPlane + px * 16, in ? src + px * kBnC : a.dy, in);
+        }
+        ld.next(a.w, a.h);
+      }
+      cp_async_commit();
+      const int e = t - (kWgStages - 1);             // the tile handed on
+      if (e >= 0) {
+        cp_async_wait<kWgStages - 1>();
+        const uint8_t *ys = sm + (e % kWgStages) * kWgStage + kCvX + (tid & 3) * kWgPlane;
+#pragma unroll
+        for (int s = 0; s < kY; ++s) {
+          const uint4 v = *reinterpret_cast<const uint4 *>(ys + ((tid >> 2) + s * (kWgThreads / 4)) * 16);
+          const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            dbp[2 * q] += __uint_as_float(u[q] << 16);
+            dbp[2 * q + 1] += __uint_as_float(u[q] & 0xffff0000u);
+          }
+        }
+        fence_async_smem();
+        bn_arrive(&full[e % kWgStages]);
+      }
+    }
+    cp_async_wait<0>();
+  } else {
+    constexpr uint32_t idesc = idesc_bf16(128, 32, true);
+    const uint32_t leader = elect_one();
+    int issued = 0;
+    for (int t = 0; t < nt; ++t) {
+      if (!wait(&full[t % kWgStages], t / kWgStages)) break;
+      tc_fence_after();
+      const uint32_t x_0 = smem_u32(sm) + (t % kWgStages) * kWgStage;
+      const uint64_t xd = sdesc(x_0, 128, kCvPlane), yd = sdesc(x_0 + kCvX, 128, kWgPlane);
+      // the three accumulators in turn: MMAs into one accumulator follow each other slower
+#pragma unroll
+      for (int s = 0; s < kCvM / 16; ++s)
+#pragma unroll
+        for (int kx = 0; kx < 3; ++kx)
+          umma_bf16(tmem + 32 * kx, sdesc_at(xd, kx * 16 + s * 256), sdesc_at(yd, s * 256), idesc,
+                    (t > 0 || s > 0) ? 1u : 0u, leader);
+      umma_commit(&empty[t % kWgStages], leader);
+      issued = t + 1;
+    }
+    // every MMA has completed before the accumulators are read and freed
+    for (int t = max(0, issued - kWgStages); t < issued; ++t) wait(&empty[t % kWgStages], t / kWgStages);
   }
+  tc_fence_before();
+  ok = __syncthreads_and(ok) != 0;
+  tc_fence_after();
   float *part = a.part + (size_t)blockIdx.x * kWgPart;
+  if (warp < 3) {                                    // accumulator rows ky * 32 + ci: warp ky, lane ci
 #pragma unroll 1
-  for (int t = 0; t < 3; ++t) {
-    float v[32];
-    if (ok && issued > 0) {
-      tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + 32 * t, v);
-    } else {
+    for (int kx = 0; kx < 3; ++kx) {
+      float v[32];
+      if (ok) {   // (a CTA has at least one tile)
+        tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + 32 * kx, v);
+      } else {
 #pragma unroll
-      for (int c = 0; c < 32; ++c) v[c] = 0.0f;
-    }
-    const int m = 128 * t + warp * 32 + lane;   // (tap, ci) row
-    if (m < kBnK) {
+        for (int c = 0; c < 32; ++c) v[c] = 0.0f;
+      }
 #pragma unroll
-      for (int c = 0; c < 32; ++c) part[c * kBnK + m] = v[c];
+      for (int c = 0; c < 32; ++c) part[c * kBnK + (warp * 3 + kx) * kBnC + lane] = v[c];
     }
   }
-  // bias gradient: each warp's sums, then the four warps in order
-  __shared__ float dbw[4][32];
+  // bias gradient: each warp's sums per chunk, then the warps in order
+  __shared__ float dbw[kWgThreads / 32][32];
 #pragma unroll
-  for (int c = 0; c < 32; ++c) {
+  for (int c = 0; c < 8; ++c) {
     float s = dbp[c];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) dbw[warp][c] = s;
+    for (int o = 4; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane < 4 && warp < kWgLoad) dbw[warp][lane * 8 + c] = s;
   }
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x < 32)
-    part[kBnK * 32 + threadIdx.x] = ((dbw[0][threadIdx.x] + dbw[1][threadIdx.x]) + dbw[2][threadIdx.x]) + dbw[3][threadIdx.x];
+  if (tid < 32) {
+    float s = dbw[0][tid];
+    for (int q = 1; q < kWgThreads / 32; ++q) s += dbw[q][tid];
+    part[kBnK * 32 + tid] = s;
+  }
   if (warp == 0) tmem_dealloc(tmem, 128);
 }
 
@@ -688,12 +808,19 @@ extern "C" sgmf_status sgmf_bn_conv(int n, int h, int w, const uint16_t *x, cons
   return bn_launch(cudaGetLastError(), "sgmf_bn_conv");
 }
 
-// dw / db += the partials of `ctas` CTAs, added in CTA order
-__global__ void __launch_bounds__(256) k_bn_wgrad_sum(const float *__restrict__ part, int ctas, float *dw, float *db) {
-  const int o = blockIdx.x * blockDim.x + threadIdx.x;
-  if (o >= kWgPart) return;
+// dw / db += the partials of `ctas` CTAs: 32 outputs a CTA, 32 slices of the
+// partials each (slice q takes CTAs q, q + 32, ..), added in slice order
+__global__ void __launch_bounds__(1024) k_bn_wgrad_sum(const float *__restrict__ part, int ctas, float *dw, float *db) {
+  __shared__ float slice[32][33];
+  const int l = threadIdx.x & 31, q = threadIdx.x >> 5, o = blockIdx.x * 32 + l;
+  static_assert(kWgPart % 32 == 0, "whole CTAs");
   float s = 0.0f;
-  for (int b = 0; b < ctas; ++b) s += part[(size_t)b * kWgPart + o];
+#pragma unroll 8
+  for (int b = q; b < ctas; b += 32) s += part[(size_t)b * kWgPart + o];
+  slice[q][l] = s;
+  __syncthreads();
+  if (q != 0) return;
+  for (int i = 1; i < 32; ++i) s += slice[i][l];
   if (o < kBnK * 32)
     dw[o] += s;
   else
@@ -708,8 +835,7 @@ extern "C" sgmf_status sgmf_bn_wgrad(int n, int h, int w, const uint16_t *x, con
     return cudaFuncSetAttribute(k_bn_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
   });
   if (ea != cudaSuccess) return bn_launch(ea, "sgmf_bn_wgrad attribute");
-  const long long P = (long long)n * h * w;
-  const long long nchunk = (P + 127) / 128;
+  const long long nchunk = (long long)n * h * ((w + kCvM - 1) / kCvM);   // tiles
   const int chunks = (int)((nchunk + kWgMaxCtas - 1) / kWgMaxCtas);
   const unsigned grid = (unsigned)((nchunk + chunks - 1) / chunks);   // <= kWgMaxCtas
   float *part = nullptr;
@@ -717,10 +843,10 @@ extern "C" sgmf_status sgmf_bn_wgrad(int n, int h, int w, const uint16_t *x, con
   if (e != cudaSuccess) return bn_launch(e, "sgmf_bn_wgrad scratch");
   BnWgradArgs a{n, h, w, chunks, x, dy, part, err};
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  k_bn_wgrad<<<grid, 128, kWgSmem, s>>>(a);
+  k_bn_wgrad<<<grid, kWgThreads + 32, kWgSmem, s>>>(a);
   e = cudaGetLastError();
   if (e != cudaSuccess) return bn_launch(e, "sgmf_bn_wgrad");
-  k_bn_wgrad_sum<<<(kWgPart + 255) / 256, 256, 0, s>>>(part, (int)grid, dw, db);
+  k_bn_wgrad_sum<<<kWgPart / 32, 1024, 0, s>>>(part, (int)grid, dw, db);
   return bn_launch(cudaGetLastError(), "sgmf_bn_wgrad");
 }
 
