@@ -108,7 +108,7 @@ def pipeline_roofline(rates: dict, sm_mhz: float, hbm_gbs: float, V: int, N: int
 # the files that define and launch it and every header they include (the
 # shared header and the API file that sizes the buffers go with every one)
 AGG_SOURCES = ("sgmf_sweep", "sgmf_lines", "sgmf_rows", "sgmf_wta", "sgmf_lanes", "sgmf_aggregate", "sgmf_agg_cpl",
-               "sgmf_check", "sgmf_band_")
+               "sgmf_check")
 KERNEL_SOURCES = {
     "agg_lines": AGG_SOURCES, "agg_sweep": AGG_SOURCES, "agg_rows_wta": AGG_SOURCES,
     "ingest": ("sgmf_front", "sgmf_cost"), "census": ("sgmf_front", "sgmf_cost"),

@@ -401,8 +401,8 @@ sgmf_status sgmf_set_gate(sgmf_ctx *c, const int *gate, int run);
 /* ---- Launch tuning (no counterpart in the paper) -----------------------
  * Launch shapes only: every choice gives bit-identical results. */
 typedef struct {
-    int32_t line_warps;   /* warps per CTA of the vertical/diagonal line kernels
-                             (each warp walks two lines): 1, 2, 4 (default) or 8 */
+    int32_t line_warps;   /* warps per CTA of the line kernels (each warp walks
+                             four lines in one direction): 1, 2, 4 (default) or 8 */
     int32_t cost_px;      /* the cost kernel takes row segments of at most
                              8 x cost_px pixels per CTA: 32, 64 or 128 (default;
                              segments of up to 1024 pixels) */
@@ -410,12 +410,13 @@ typedef struct {
                              row-synchronous sweeps of a thread-block cluster per
                              frame (one launch) instead of the three line kernels
                              (line_warps is then unused).  0 (default) or 1; 1 needs
-                             a row of at most 16 CTAs x 128 pixels (Dp <= 128; banded:
-                             x 160) or 16 x 80 pixels (Dp > 128) and
+                             a row of at most 16 CTAs x 128 pixels (Dp <= 128) or
+                             16 x 80 pixels (Dp > 128; banded: 16 x 160) and
                              a device that can place such a cluster (the context
                              picks the cluster size that keeps the most CTAs
                              resident), and is refused otherwise; it takes effect
-                             with 8 paths. */
+                             with 8 paths on a plain context (a banded one walks
+                             lines, which is faster there). */
     int32_t parts;        /* with the sweep: 1 (default) runs a batch in parts of one
                              sweep wave, each part's row kernel on a second stream
                              beside the next part's sweep; 0 runs the whole batch

@@ -1,4 +1,4 @@
 // sgmf_agg_cpl16.cu -- aggregation kernels with 16 disparity cells per lane (Dp = 128).
 #include "sgmf_sweep.cuh"
 
-SGMF_OCT_INSTANTIATE(16)
+SGMF_AGG_INSTANTIATE(16)

@@ -1,4 +1,4 @@
 // sgmf_agg_cpl24.cu -- aggregation kernels with 24 disparity cells per lane (Dp = 192).
 #include "sgmf_sweep.cuh"
 
-SGMF_OCT_INSTANTIATE(24)
+SGMF_AGG_INSTANTIATE(24)

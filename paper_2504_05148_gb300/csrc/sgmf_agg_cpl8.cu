@@ -1,4 +1,4 @@
 // sgmf_agg_cpl8.cu -- aggregation kernels with 8 disparity cells per lane (Dp = 64).
 #include "sgmf_sweep.cuh"
 
-SGMF_OCT_INSTANTIATE(8)
+SGMF_AGG_INSTANTIATE(8)

@@ -36,7 +36,7 @@ struct sgmf_ctx {
   static constexpr int kMaxParts = 8;
   cudaStream_t side = nullptr;
   cudaEvent_t ev_part[kMaxParts] = {};
-  cudaEvent_t ev_rows = nullptr, ev_in = nullptr;
+  cudaEvent_t ev_rows = nullptr;
   size_t bytes = 0;
   std::string err;
   // device staging for sgmf_compute_host
@@ -207,10 +207,8 @@ static void free_all(sgmf_ctx *c) {
     if (c->ev_part[i]) cudaEventDestroy(c->ev_part[i]);
     c->ev_part[i] = nullptr;
   }
-  for (cudaEvent_t *e : {&c->ev_rows, &c->ev_in}) {
-    if (*e) cudaEventDestroy(*e);
-    *e = nullptr;
-  }
+  if (c->ev_rows) cudaEventDestroy(c->ev_rows);
+  c->ev_rows = nullptr;
   if (c->side) cudaStreamDestroy(c->side);
   c->side = nullptr;
 }
@@ -246,6 +244,8 @@ static cudaError_t side_stream(cudaStream_t *s) {
   if (e != cudaSuccess) return e;
   return cudaStreamCreateWithPriority(s, cudaStreamNonBlocking, kSidePriority ? greatest : least);
 }
+
+constexpr int kMaxBandSweepRow = 2560;
 
 static sgmf_status create_ctx(int width, int height, int max_disp, int max_batch, int band, sgmf_ctx **out) {
   if (!out) return fail(nullptr, SGMF_ERR_ARG, "sgmf_create: out is NULL");
@@ -327,15 +327,15 @@ static sgmf_status create_ctx(int width, int height, int max_disp, int max_batch
   }
   {
     // whether the row-synchronous sweep can run this shape (8 paths); the
-    // line kernels stay the default, the sweep is a tuning choice
+    // line kernels stay the default, the sweep is a tuning choice (which a
+    // banded context takes for rows of up to kMaxBandSweepRow pixels)
     KParams kk = k;
     kk.num_paths = 8;
-    c->k.sweep_cs = agg_sweep_plan(kk, c->nb, &c->sweep_slots);
-    c->sweep_ok = c->k.sweep_cs > 0;
-    bool ok = !(c->sweep_ok && c->nb >= 2) ||
+    if (!band) c->k.sweep_cs = agg_sweep_plan(kk, c->nb, &c->sweep_slots);
+    c->sweep_ok = band ? width <= kMaxBandSweepRow : c->k.sweep_cs > 0;
+    bool ok = !(c->sweep_ok && c->nb >= 2 && !band) ||
               (side_stream(&c->side) == cudaSuccess &&
-               cudaEventCreateWithFlags(&c->ev_rows, cudaEventDisableTiming) == cudaSuccess &&
-               cudaEventCreateWithFlags(&c->ev_in, cudaEventDisableTiming) == cudaSuccess);
+               cudaEventCreateWithFlags(&c->ev_rows, cudaEventDisableTiming) == cudaSuccess);
     for (int i = 0; ok && c->side && i < sgmf_ctx::kMaxParts; ++i)
       ok = cudaEventCreateWithFlags(&c->ev_part[i], cudaEventDisableTiming) == cudaSuccess;
     if (!ok) {
@@ -415,8 +415,11 @@ extern "C" sgmf_status sgmf_set_stream(sgmf_ctx *c, void *stream) {
 
 static bool need_boxc(const KParams &k) { return k.consistency == SGMF_CHECK_STEREO_LIDAR || k.consistency == SGMF_CHECK_LIDAR; }
 
-// the sweep runs when the tuning asks for it and the context allows it
-static bool use_sweep(const sgmf_ctx *c) { return c->k.sweep && c->k.num_paths == 8 && c->sweep_ok; }
+// The sweep runs when the tuning asks for it and the context allows it; a
+// banded context takes the tuning but walks lines all the same (1920 x 1080,
+// bands of 64, 8 frames: 7.5 ms a call, 8.4 with a sweep on these lane groups in
+// parts, 8.9 with the 16-lane sweep and rows they replaced).
+static bool use_sweep(const sgmf_ctx *c) { return c->k.sweep && c->k.num_paths == 8 && c->sweep_ok && !c->k.band; }
 
 // Frames per part when a sweep batch of n frames goes through in parts (0:
 // one part).  A part's row kernel and check run on the side stream beside
@@ -447,9 +450,10 @@ static int front_launches(const KParams &k) {
 
 extern "C" int sgmf_launches_per_compute(const sgmf_ctx *c) {
   if (!c) return 0;
-  // front stages, one line launch per family (one sweep launch for all six directions), rows, consistency
-  // (a sweep batch in parts launches the sweep, rows and check once per part; counted for a full batch)
-  const int agg = (c->k.num_paths == 8 ? (use_sweep(c) ? 1 : 3) : 1) + 2;
+  // front stages, then the sweep, rows and check (once per part of a batch in
+  // parts; counted for a full batch), or one launch per line family, the rows
+  // among them (two where their costs are u16), and the winner kernel, which checks
+  const int agg = use_sweep(c) ? 3 : (c->k.num_paths == 8 ? 3 : 1) + (c->spill8 ? 1 : 2) + 1;
   int parts = 1;
   if (use_sweep(c) && sweep_part(c, c->nb) > 0) {
     const int m = sweep_part(c, c->nb);
@@ -533,6 +537,49 @@ static sgmf_status front_stages(sgmf_ctx *c, int f0, int nf, const uint8_t *left
   return SGMF_OK;
 }
 
+// What follows the cost volume (and, with the sweep, the sweep) for the nf
+// frames of b on stream s, down to the output.
+static sgmf_status finish(sgmf_ctx *c, const KParams &ka, const Buffers &b, int nf, int16_t *out, cudaStream_t s) {
+  if (ka.sweep) {
+    TIMED(c, "agg_rows_wta", s, launch_agg_rows(ka, b, nf, c->spill8, s));
+    TIMED(c, "consistency", s, launch_consistency(c->k, b, nf, out, s));
+    return SGMF_OK;
+  }
+  // every direction's vectors; what is left needs no walk
+  TIMED(c, "agg_lines", s, launch_agg_lines(ka, b, nf, c->spill8, s));
+  TIMED(c, "agg_rows_wta", s, launch_agg_wta(ka, b, nf, c->spill8, out, s));
+  return SGMF_OK;
+}
+
+// Aggregation, winners and check of the n frames whose cost volume is made.
+// A sweep batch goes through in parts of m frames: part i's sweep on the
+// context's stream, then the rest of it on the side stream while part i + 1 is
+// in the sweep; the context's stream goes on after the last part's.  (Running
+// the later parts' front stages on the side stream beside the first part's
+// sweep was measured twice and gave nothing: 8.17-8.24 against 8.20 ms for 32
+// KITTI frames, and 3 % slower at 64; the sweep slows by what they save.)
+static sgmf_status aggregate(sgmf_ctx *c, int n, int16_t *out, cudaStream_t s) {
+  const KParams ka = agg_params(c);
+  const int m = ka.sweep ? sweep_part(c, n) : 0;
+  if (m == 0) {
+    if (ka.sweep) TIMED(c, "agg_sweep", s, launch_agg_sweep(ka, c->b, n, s));
+    return finish(c, ka, c->b, n, out, s);
+  }
+  const size_t px = frame_px(c->k);
+  for (int i = 0, f0 = 0; f0 < n; ++i, f0 += m) {
+    const int nf = std::min(m, n - f0);
+    const Buffers bp = frame_view(c->k, c->b, f0);
+    TIMED(c, "agg_sweep", s, launch_agg_sweep(ka, bp, nf, s));
+    CUDA_TRY(c, cudaEventRecord(c->ev_part[i], s));
+    CUDA_TRY(c, cudaStreamWaitEvent(c->side, c->ev_part[i], 0));
+    const sgmf_status st = finish(c, ka, bp, nf, out + f0 * px, c->side);
+    if (st != SGMF_OK) return st;
+  }
+  CUDA_TRY(c, cudaEventRecord(c->ev_rows, c->side));
+  CUDA_TRY(c, cudaStreamWaitEvent(s, c->ev_rows, 0));
+  return SGMF_OK;
+}
+
 extern "C" sgmf_status sgmf_compute_batch(sgmf_ctx *c, int n, const uint8_t *left, const uint8_t *right,
                                           const float *lidar, int16_t *out) {
   if (!c) return SGMF_ERR_ARG;
@@ -540,48 +587,10 @@ extern "C" sgmf_status sgmf_compute_batch(sgmf_ctx *c, int n, const uint8_t *lef
   if (n < 1 || n > c->nb)
     return fail(c, SGMF_ERR_ARG, "sgmf_compute_batch: need 1 <= n <= %d frames (got %d)", c->nb, n);
   if (c->k.band) return fail(c, SGMF_ERR_ARG, "sgmf_compute: a banded context needs sgmf_compute_banded");
-  const KParams &k = c->k;
-  const size_t px = (size_t)k.W * k.H;
-  cudaStream_t s = c->stream;
   prof_reset(c);
-  const KParams ka = agg_params(c);
-  const int m = ka.sweep ? sweep_part(c, n) : 0;
-  if (m > 0) {
-    // Parts of m frames after the front stages of all n: part i's sweep on
-    // the context's stream, then its row kernel and check on the side
-    // stream while part i + 1 is in the sweep; the context's stream goes on
-    // after the last part's check.  (Running the later parts' front stages
-    // on the side stream beside the first part's sweep was measured twice
-    // and gave nothing: 8.17-8.24 against 8.20 ms for 32 KITTI frames, and
-    // 3 % slower at 64; the sweep slows by what the front stages save.)
-    sgmf_status st = front_stages(c, 0, n, left, right, lidar, true, s);
-    if (st != SGMF_OK) return st;
-    for (int i = 0, f0 = 0; f0 < n; ++i, f0 += m) {
-      const int nf = std::min(m, n - f0);
-      const Buffers bp = frame_view(k, c->b, f0);
-      TIMED(c, "agg_sweep", s, launch_agg_sweep(ka, bp, nf, s));
-      CUDA_TRY(c, cudaEventRecord(c->ev_part[i], s));
-      CUDA_TRY(c, cudaStreamWaitEvent(c->side, c->ev_part[i], 0));
-      TIMED(c, "agg_rows_wta", c->side, launch_agg_rows(ka, bp, nf, c->spill8, c->side));
-      TIMED(c, "consistency", c->side, launch_consistency(k, bp, nf, out + f0 * px, c->side));
-    }
-    CUDA_TRY(c, cudaEventRecord(c->ev_rows, c->side));
-    CUDA_TRY(c, cudaStreamWaitEvent(s, c->ev_rows, 0));
-  } else {
-    sgmf_status st = front_stages(c, 0, n, left, right, lidar, true, s);
-    if (st != SGMF_OK) return st;
-    if (ka.sweep)
-      TIMED(c, "agg_sweep", s, launch_agg_sweep(ka, c->b, n, s));
-    else
-      TIMED(c, "agg_lines", s, launch_agg_lines(ka, c->b, n, c->spill8, s));
-    if (!ka.sweep && c->spill8) {
-      // the line kernels walked the rows too: what is left needs no walk
-      TIMED(c, "agg_rows_wta", s, launch_agg_wta(ka, c->b, n, out, s));
-    } else {
-      TIMED(c, "agg_rows_wta", s, launch_agg_rows(ka, c->b, n, c->spill8, s));
-      TIMED(c, "consistency", s, launch_consistency(k, c->b, n, out, s));
-    }
-  }
+  sgmf_status st = front_stages(c, 0, n, left, right, lidar, true, c->stream);
+  if (st == SGMF_OK) st = aggregate(c, n, out, c->stream);
+  if (st != SGMF_OK) return st;
   c->computed = true;
   c->last_n = n;
   return SGMF_OK;
@@ -739,11 +748,8 @@ extern "C" sgmf_status sgmf_debug_stage(sgmf_ctx *c, int stage, void *dst, size_
     case SGMF_STAGE_SUM: {
       const bool u16 = stage == SGMF_STAGE_SUM;
       const void *src = u16 ? static_cast<const void *>(c->b.dbg_sum) : c->b.cost;
-      if (k.band) {   // banded: [H][W][band], cell j = disparity lo_p + j
-        CUDA_TRY(c, cudaMemcpy(dst, src, need, cudaMemcpyDeviceToHost));
-        break;
-      }
-      // full range: Dp cells a pixel in group-lane order
+      // Dp cells a pixel in group-lane order (banded: Dp = band, cell j = disparity lo_p + j)
+      const int nd = k.band ? k.band : k.D;
       const size_t es = u16 ? 2 : 1;
       std::vector<uint8_t> tmp(n * k.Dp * es);
       CUDA_TRY(c, cudaMemcpy(tmp.data(), src, tmp.size(), cudaMemcpyDeviceToHost));
@@ -751,8 +757,8 @@ extern "C" sgmf_status sgmf_debug_stage(sgmf_ctx *c, int stage, void *dst, size_
       for (int m = 0; m < k.Dp; ++m) cell[m] = lane_order_cell(k.Dp, u16, m);
       for (size_t p = 0; p < n; ++p)
         for (int m = 0; m < k.Dp; ++m)
-          if (cell[m] < k.D)
-            memcpy(static_cast<uint8_t *>(dst) + (p * k.D + cell[m]) * es, &tmp[(p * k.Dp + m) * es], es);
+          if (cell[m] < nd)
+            memcpy(static_cast<uint8_t *>(dst) + (p * nd + cell[m]) * es, &tmp[(p * k.Dp + m) * es], es);
       break;
     }
   }
@@ -920,33 +926,8 @@ extern "C" sgmf_status sgmf_compute_banded_back(sgmf_ctx *c, int n, const int16_
   cudaStream_t s = c->stream;
   TIMED(c, "band_clamp", s, launch_band_clamp(k, c->b, n, band_lo, s));
   TIMED(c, "cost", s, launch_cost_banded(k, c->b, n, s));
-  const KParams ka = agg_params(c);
-  const int m = ka.sweep ? sweep_part(c, n) : 0;
-  if (m > 0) {
-    // parts of m frames: part i's row kernel and check on the side stream
-    // beside part i + 1's sweep (as in sgmf_compute_batch)
-    const size_t px = (size_t)k.W * k.H;
-    CUDA_TRY(c, cudaEventRecord(c->ev_in, s));
-    CUDA_TRY(c, cudaStreamWaitEvent(c->side, c->ev_in, 0));
-    for (int i = 0, f0 = 0; f0 < n; ++i, f0 += m) {
-      const int nf = std::min(m, n - f0);
-      const Buffers bp = frame_view(k, c->b, f0);
-      TIMED(c, "agg_sweep", s, launch_agg_sweep(ka, bp, nf, s));
-      CUDA_TRY(c, cudaEventRecord(c->ev_part[i], s));
-      CUDA_TRY(c, cudaStreamWaitEvent(c->side, c->ev_part[i], 0));
-      TIMED(c, "agg_rows_wta", c->side, launch_agg_rows(ka, bp, nf, c->spill8, c->side));
-      TIMED(c, "consistency", c->side, launch_consistency(k, bp, nf, out + f0 * px, c->side));
-    }
-    CUDA_TRY(c, cudaEventRecord(c->ev_rows, c->side));
-    CUDA_TRY(c, cudaStreamWaitEvent(s, c->ev_rows, 0));
-  } else {
-    if (ka.sweep)
-      TIMED(c, "agg_sweep", s, launch_agg_sweep(ka, c->b, n, s));
-    else
-      TIMED(c, "agg_lines", s, launch_agg_lines(ka, c->b, n, c->spill8, s));
-    TIMED(c, "agg_rows_wta", s, launch_agg_rows(ka, c->b, n, c->spill8, s));
-    TIMED(c, "consistency", s, launch_consistency(k, c->b, n, out, s));
-  }
+  const sgmf_status st = aggregate(c, n, out, s);
+  if (st != SGMF_OK) return st;
   c->computed = true;
   c->last_n = n;
   c->front_n = 0;

@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(256) k_cost_banded(KParams k, Buffers b0, cons
   const int j0 = DPL * lane;                      // the lane's first band cell
   // every pixel of the CTA has x - d >= 0 for all its band cells
   const bool inner = x0 >= lo_max + B - 1;
-  uint8_t *out = b.cost + (rowp + x0) * B + j0;
+  uint8_t *out = b.cost + (rowp + x0) * B;
   for (int xb = P * warp; xb < npx; xb += P * nwarp) {
     const int lo = lo_s[xb >> kBandTileLog];
     // cR(x - lo - j) of pixel xb + u and cell j = j0 + i is entry jlo + DPL - 1 + u - i
@@ -162,9 +162,7 @@ __global__ void __launch_bounds__(256) k_cost_banded(KParams k, Buffers b0, cons
           o[u][i] = tab_s[cls * 64 + h];
         }
     }
-#pragma unroll
-    for (int u = 0; u < P; ++u)
-      if (xb + u < npx) store_cost_bytes<DPL>(out + (size_t)(xb + u) * B, o[u]);
+    store_cost_quad<DPL>(out + (size_t)xb * B, o, lane, npx - xb);
   }
 }
 

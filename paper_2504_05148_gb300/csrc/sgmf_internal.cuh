@@ -7,7 +7,7 @@
 //   box-OR masks    u32    [F][MW][H][W]   bit d of word-plane d/32 set when a
 //                                           sparse disparity of the window is d
 //   cost C-bar      uint8  [F][H][W][Dp]   Dp = 32 * DPL >= D, cells d >= D hold 0;
-//                                           full range: cells in group-lane order (sgmf_lanes.cuh)
+//                                           cells in group-lane order (sgmf_lanes.cuh)
 //   partial sums    u16    [F][H][W][Dp]   one per line family (vertical, two diagonals)
 //   spills          uint8/u16 [F][4][line][pos][Dp]  first-direction path costs of a line
 // F is the number of frames a context holds (its batch capacity); every
@@ -127,28 +127,8 @@ struct CostVec {
   using V = typename std::conditional<VL * sizeof(CT) == 16, uint4, uint2>::type;
 };
 
-template <int DPL>
-__device__ __forceinline__ void store_cost_bytes(uint8_t *o, const uint32_t (&b)[DPL]) {
-  uint32_t w[(DPL + 3) / 4];
-#pragma unroll
-  for (int j = 0; j < DPL / 4; ++j)
-    w[j] = prmt(prmt(b[4 * j], b[4 * j + 1], 0x1140), prmt(b[4 * j + 2], b[4 * j + 3], 0x1140), 0x5410);
-  if constexpr (DPL == 2) {
-    *reinterpret_cast<uint16_t *>(o) = (uint16_t)prmt(b[0], b[1], 0x1140);
-  } else if constexpr (DPL == 4) {
-    *reinterpret_cast<uint32_t *>(o) = w[0];
-  } else if constexpr (DPL == 6) {   // 2-byte aligned
-    uint16_t *q = reinterpret_cast<uint16_t *>(o);
-    q[0] = (uint16_t)prmt(b[0], b[1], 0x1140);
-    q[1] = (uint16_t)prmt(b[2], b[3], 0x1140);
-    q[2] = (uint16_t)prmt(b[4], b[5], 0x1140);
-  } else {
-    *reinterpret_cast<uint2 *>(o) = make_uint2(w[0], w[1]);
-  }
-}
-
-// Four pixels' bytes into the full-range volume, whose cells lie in the order of
-// the aggregation kernels' lanes (sgmf_lanes.cuh): with CPL = 4 DPL cells a
+// Four pixels' bytes into the cost volume, whose cells lie in the order of the
+// aggregation kernels' lanes (sgmf_lanes.cuh): with CPL = 4 DPL cells a
 // group lane, cell w of a group lane and cell w + CPL / 2 are neighbours.  The
 // cost kernel's lanes 4 j .. 4 j + 3 hold group lane j's cells; lanes s and s + 2
 // of them hold the two halves of the same pairs: the first takes both halves
@@ -217,7 +197,7 @@ __device__ __forceinline__ void store_cost_quad(uint8_t *out, const uint32_t (&b
 }
 
 // cell of the group-lane order's position m in the byte form (u16 = false) or
-// the u16 form of a full-range vector of Dp cells (host: debug copies)
+// the u16 form of a vector of Dp cells (host: debug copies)
 inline int lane_order_cell(int Dp, bool u16, int m) {
   const int CPL = Dp / 8, NW = CPL / 2;
   int j, b;
@@ -371,10 +351,12 @@ cudaError_t launch_boxor_cols(const KParams &k, int nf, const uint32_t *src, uin
                               const int *gate = nullptr);
 cudaError_t launch_semidense(const KParams &k, const Buffers &b, int nf, cudaStream_t s);
 cudaError_t launch_cost(const KParams &k, const Buffers &b, int nf, cudaStream_t s);
-cudaError_t launch_agg_lines(const KParams &k, const Buffers &b, int nf, bool spill8, cudaStream_t s);
-cudaError_t launch_agg_rows(const KParams &k, const Buffers &b, int nf, bool spill8, cudaStream_t s);
-// S, d*, d' and the check from the line walks' byte vectors (rows among them)
-cudaError_t launch_agg_wta(const KParams &k, const Buffers &b, int nf, int16_t *out, cudaStream_t s);
+// the line walks of every direction; bytes: path costs fit a byte
+cudaError_t launch_agg_lines(const KParams &k, const Buffers &b, int nf, bool bytes, cudaStream_t s);
+// behind the sweep: the row directions, S, d* and d'
+cudaError_t launch_agg_rows(const KParams &k, const Buffers &b, int nf, bool bytes, cudaStream_t s);
+// S, d*, d' and the check from the walks' vectors
+cudaError_t launch_agg_wta(const KParams &k, const Buffers &b, int nf, bool bytes, int16_t *out, cudaStream_t s);
 // the six vertical/diagonal directions as two cluster sweeps (k.sweep, clusters of
 // k.sweep_cs CTAs); plan: the cluster size for the context's shape and batch capacity nb on
 // this device, 0 if none, and in *slots the number of such clusters the device holds at once

@@ -229,18 +229,32 @@ struct StepConsts {
   uint32_t dpx2;   // (P2 - P1) in both halves
 };
 
-// One step of Eq. 2 for the lane's words.  mm = min_k L(p - r, k) in both
-// halves.  lo_edge / hi_edge are 0xffff in the missing neighbour's half on the
-// first / last lane of the group (L(-1), L(Dp) only enter a min), else 0.
-template <int NW>
+// The group's outer neighbours, as bits ORed into the first / last lane's words:
+// 0xffff in the missing neighbour's half (L(-1), L(Dp) only enter a min).  On the
+// bands the neighbour's half is cleared first (keep) and may hold the previous
+// pixel's cell just outside the current band (band_shift).
+struct Edges {
+  uint32_t lo, hi;
+};
+__device__ __forceinline__ Edges no_neighbours(int lig) {
+  return {lig == 0 ? 0xffffu : 0u, lig == kGL - 1 ? 0xffff0000u : 0u};
+}
+
+// One step of Eq. 2 for the lane's words.  mm = min_k L(p - r, k) in both halves.
+template <int NW, bool BANDED = false>
 __device__ __forceinline__ void step(uint32_t (&L)[NW], const uint32_t (&C)[NW], uint32_t mm, const StepConsts &sc,
-                                     uint32_t lo_edge, uint32_t hi_edge) {
+                                     Edges e, int lig = 0) {
   const uint32_t below = __shfl_up_sync(kAll, L[NW - 1], 1, kGL);
   const uint32_t above = __shfl_down_sync(kAll, L[0], 1, kGL);
   // below the first word: (cell CPL - 1 of the lane below, own cell NW - 1);
   // above the last: (own cell NW, cell 0 of the lane above)
-  uint32_t left = prmt(below, L[NW - 1], 0x5432) | lo_edge;
-  const uint32_t last = prmt(L[0], above, 0x5432) | hi_edge;
+  uint32_t left = prmt(below, L[NW - 1], 0x5432), last = prmt(L[0], above, 0x5432);
+  if constexpr (BANDED) {
+    left &= lig == 0 ? 0xffff0000u : 0xffffffffu;
+    last &= lig == kGL - 1 ? 0xffffu : 0xffffffffu;
+  }
+  left |= e.lo;
+  last |= e.hi;
   const uint32_t cap = mm + sc.dpx2;           // m + P2 - P1 per half
   const uint32_t negmm = 0u - mm;
 #pragma unroll
@@ -283,6 +297,42 @@ __device__ __forceinline__ uint32_t group_min_u32(uint32_t v) {
 #pragma unroll
   for (int s = 1; s < kGL; s *= 2) v = min(v, __shfl_xor_sync(kAll, v, s));
   return v;
+}
+
+// ---- disparity bands (banded mode, not in the paper) -----------------------------
+// In banded mode cell j of pixel p stands for disparity lo_p + j, with lo_p
+// constant on 8 x 8 pixel tiles.  Where the band start changes by delta along a
+// path, the previous pixel's path costs are re-indexed: cell j takes old cell
+// j + delta, and the cells that have no old counterpart become absent (kInf,
+// above every real path cost, so they only ever lose a min).  m of the previous
+// pixel stays the min over its own band.  The recursion on the bands is the
+// exact dynamic program of Eq. 1 with each pixel's labels restricted to its
+// band, so the previous pixel's cell just below the new band (old cell
+// delta - 1, for delta > 0) or just above it (old cell B + delta, for
+// delta < 0) is still the d-1 / d+1 neighbour of the new band's end cell: the
+// shift hands it to the next step as the end lane's edge.
+//
+// Runs on all 32 lanes: a group with delta = 0 rewrites its cells in place.
+// buf: the group's shared scratch, 8 NW words.
+template <int NW>
+__device__ __forceinline__ Edges band_shift(uint32_t (&L)[NW], int delta, uint32_t *buf, int lig) {
+  constexpr int CPL = 2 * NW, B = kGL * CPL;
+#pragma unroll
+  for (int i = 0; i < NW; ++i) buf[lig * NW + i] = L[i];
+  __syncwarp();
+  const uint16_t *cells = reinterpret_cast<const uint16_t *>(buf);
+  auto old = [&](int c, uint32_t absent) -> uint32_t {   // old cell c
+    const int r = c % CPL;
+    return (unsigned)c < (unsigned)B ? (uint32_t)cells[2 * (c / CPL * NW + r % NW) + r / NW] : absent;
+  };
+#pragma unroll
+  for (int i = 0; i < NW; ++i) {
+    const int c = lig * CPL + i + delta;
+    L[i] = old(c, kInf) | old(c + NW, kInf) << 16;
+  }
+  const uint32_t v = old(lig == 0 ? delta - 1 : B + delta, 0xffffu);
+  __syncwarp();
+  return {lig == 0 ? v : 0u, lig == kGL - 1 ? v << 16 : 0u};
 }
 
 // Sub-pixel disparity in 1/16 px: the vertex of the parabola through sm =

@@ -23,6 +23,8 @@
 // (6.3 TB/s: the DRAM bound).  8 steps ahead: 195 us for one frame, 16: 181.
 #pragma once
 
+#include <algorithm>
+
 #include "sgmf_lanes.cuh"
 
 namespace sgmf {
@@ -35,16 +37,20 @@ struct LineArgs {
   size_t dst_frame[2];    // bytes from one frame to the next
   StepConsts sc;
   const int *gate;        // per-frame gate words of the launch's frames, or null
+  int dir;                // the direction of a launch of one direction
+  const int16_t *lo;      // banded mode: band starts per tile, [frame][th][tw]
 };
 
 // A position on a line: its pixel index p, column x, and whether the path
 // restarts there.  Wrapping at x = xw the line goes on, a new path, at xs.
 template <int FAM>
 struct LinePos {
-  int p, x;
+  int p, x, y;                   // (y: banded mode)
   bool start;
-  __device__ __forceinline__ void next(int dp, int dx, int xw, int xs, int W) {
+  __device__ __forceinline__ void next(int dp, int dx, int dy, int xw, int xs, int W) {
     p += dp;
+    y += dy;
+    if constexpr (FAM == 3) x += dx;
     if constexpr (FAM == 1 || FAM == 2) {
       x += dx;
       start = x == xw;
@@ -56,9 +62,12 @@ struct LinePos {
 
 constexpr int kLineAhead = 16;   // steps copied ahead (a multiple of the four unrolled)
 
-template <int CPL, bool S8, int FAM>
+// ADD: the vector of the pixel's other direction, there already, is added (u16
+// rows: one vector for both).  BANDED: on the bands (no padding cells).
+template <int CPL, bool S8, int FAM, bool BANDED, bool ADD>
 __global__ void __launch_bounds__(256) k_lines(const __grid_constant__ LineArgs a) {
-  constexpr int NW = CPL / 2, Dp = kGL * CPL, A = kLineAhead, U = 4, kSlot = 32 * CPL;
+  constexpr int NW = CPL / 2, Dp = kGL * CPL, A = kLineAhead, U = 4, k8 = 32 * CPL, kSlot = k8 * (ADD ? 3 : 1);
+  static_assert(!(ADD && S8), "byte vectors have a place each");
   extern __shared__ __align__(128) uint8_t smem[];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int f = blockIdx.z;
@@ -70,25 +79,27 @@ __global__ void __launch_bounds__(256) k_lines(const __grid_constant__ LineArgs 
     asm volatile("griddepcontrol.wait;" ::: "memory");
     return;
   }
-  const bool up = blockIdx.y != 0;
+  const bool up = gridDim.y == 1 ? a.dir != 0 : blockIdx.y != 0;
   const int line = min(line0 + grp, lines - 1);  // a group past the last line repeats it and stores nothing
   const bool act = line0 + grp < lines;
   const uint8_t *cost = a.cost + f * frame_cells(a.k) + lig * Vec8<CPL>::kLane;
   uint8_t *dst = a.dst[up] + f * a.dst_frame[up] + lig * VecW<CPL, S8>::kLane;
   uint8_t *ring = smem + warp * (A * kSlot);
   const uint32_t ring_s = smem_u32(ring);
-  uint32_t z[CPL / 4];
-  pad_bytes<CPL>(a.k.D, lig, z);
-  const uint32_t lo_edge = lig == 0 ? 0xffffu : 0u, hi_edge = lig == kGL - 1 ? 0xffff0000u : 0u;
+  uint32_t z[CPL / 4] = {};
+  if constexpr (!BANDED) pad_bytes<CPL>(a.k.D, lig, z);
+  const Edges none = no_neighbours(lig);
   const StepConsts sc = a.sc;
   // the first pixel and the move per step
   const int dx = FAM == 0 ? 0 : (FAM == 3 ? (up ? -1 : 1) : ((FAM == 1) != up ? 1 : -1));
+  const int dy = FAM == 3 ? 0 : (up ? -1 : 1);
   const int xw = dx > 0 ? W : -1, xs = dx > 0 ? 0 : W - 1;
   LinePos<FAM> in;
   in.start = false;                              // (the first step starts from a zero vector anyway)
   int dp;
   if constexpr (FAM == 3) {
     in.x = up ? W - 1 : 0;
+    in.y = line;
     in.p = line * W + in.x;
     dp = dx;
   } else {
@@ -97,13 +108,15 @@ __global__ void __launch_bounds__(256) k_lines(const __grid_constant__ LineArgs 
       const int x = (FAM == 1 ? line + (H - 1) : line - (H - 1)) % W;
       in.x = x < 0 ? x + W : x;
     }
-    in.p = (up ? (H - 1) * W : 0) + in.x;
+    in.y = up ? H - 1 : 0;
+    in.p = in.y * W + in.x;
     dp = (up ? -W : W) + dx;
   }
   LinePos<FAM> at = in;                          // in: next step to copy; at: next step to take
   auto copy = [&](uint32_t slot) {
     copy8<CPL>(slot, lane, cost + (size_t)(unsigned)in.p * Dp);
-    in.next(dp, dx, xw, xs, W);
+    if constexpr (ADD) copy16<CPL>(slot + k8, lane, dst + (size_t)(unsigned)in.p * (2 * Dp));
+    in.next(dp, dx, dy, xw, xs, W);
   };
 #pragma unroll 1
   for (int t = 0; t < A; ++t) {
@@ -114,17 +127,39 @@ __global__ void __launch_bounds__(256) k_lines(const __grid_constant__ LineArgs 
 #pragma unroll
   for (int w = 0; w < NW; ++w) L[w] = 0u;
   uint32_t mm = 0u;
+  // banded: the tile and band start of the step before, the group's shift scratch
+  [[maybe_unused]] const int16_t *lo = nullptr;
+  [[maybe_unused]] int tile = 0, cur = 0;
+  [[maybe_unused]] uint32_t *buf = nullptr;
+  if constexpr (BANDED) {
+    lo = a.lo + (size_t)f * a.k.th * a.k.tw;
+    tile = (at.y >> kBandTileLog) * a.k.tw + (at.x >> kBandTileLog);
+    cur = lo[tile];
+    buf = reinterpret_cast<uint32_t *>(smem + (blockDim.x >> 5) * (A * kSlot)) + (warp * kGW + grp) * (kGL * NW);
+  }
   // the next step's cost bytes are read while this step's minimum is formed
   Raw8<CPL> nxt;
   cp_wait<A - 1>();
   slot_raw8<CPL>(ring, lane, nxt);
   // a step on the bytes read before; slot: the next step's.  The copy into
   // the slot of the step itself follows (its bytes are in registers)
-  auto take = [&](const uint8_t *slot) {
+  auto take = [&](const uint8_t *slot, [[maybe_unused]] const uint8_t *own) {
     uint32_t C[NW];
     expand8<CPL>(nxt, z, C);
+    [[maybe_unused]] uint32_t other[NW];
+    if constexpr (ADD) slot16<CPL>(own + k8, lane, other);
     cp_wait<A - 2>();
     slot_raw8<CPL>(slot, lane, nxt);
+    Edges e = none;
+    if constexpr (BANDED) {
+      const int tl = (at.y >> kBandTileLog) * a.k.tw + (at.x >> kBandTileLog);
+      if (__any_sync(kAll, tl != tile)) {
+        const int now = lo[tl], delta = now - cur;
+        tile = tl;
+        cur = now;
+        if (__any_sync(kAll, delta != 0)) e = band_shift<NW>(L, delta, buf, lig);
+      }
+    }
     if constexpr (FAM == 1 || FAM == 2) {
       if (__any_sync(kAll, at.start)) {
         const uint32_t keep = at.start ? 0u : 0xffffffffu;
@@ -133,17 +168,24 @@ __global__ void __launch_bounds__(256) k_lines(const __grid_constant__ LineArgs 
         mm &= keep;
       }
     }
-    step<NW>(L, C, mm, sc, lo_edge, hi_edge);
+    step<NW, BANDED>(L, C, mm, sc, e, lig);
     mm = group_min<NW>(L);
-    if (act) VecW<CPL, S8>::put(dst + (size_t)(unsigned)at.p * (2 * Dp), L);
-    at.next(dp, dx, xw, xs, W);
+    uint8_t *o = dst + (size_t)(unsigned)at.p * (2 * Dp);
+    if constexpr (ADD) {
+#pragma unroll
+      for (int w = 0; w < NW; ++w) other[w] += L[w];
+      if (act) store_u16<CPL>(o, other);
+    } else if (act) {
+      VecW<CPL, S8>::put(o, L);
+    }
+    at.next(dp, dx, dy, xw, xs, W);
   };
   int t = 0, base = 0;                           // base: the slot of step t
   for (; t + A + U <= n; t += U) {               // U steps and the U copied into their slots all exist
     const int after = base + U * kSlot == A * kSlot ? 0 : base + U * kSlot;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      take(ring + (u + 1 < U ? base + (u + 1) * kSlot : after));
+      take(ring + (u + 1 < U ? base + (u + 1) * kSlot : after), ring + base + u * kSlot);
       copy(ring_s + base + u * kSlot);
       cp_commit();
     }
@@ -152,7 +194,7 @@ __global__ void __launch_bounds__(256) k_lines(const __grid_constant__ LineArgs 
 #pragma unroll 1
   for (; t < n; ++t) {
     const int after = base + kSlot == A * kSlot ? 0 : base + kSlot;
-    take(ring + after);                          // (past the last step: bytes never used)
+    take(ring + after, ring + base);             // (past the last step: bytes never used)
     if (t + A < n) copy(ring_s + base);
     cp_commit();
     base = after;
@@ -163,15 +205,17 @@ __global__ void __launch_bounds__(256) k_lines(const __grid_constant__ LineArgs 
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-template <int CPL, bool S8, int FAM>
-static cudaError_t launch_family(const LineArgs &a, int nf, bool overlap, cudaStream_t s) {
-  const int warps = a.k.line_warps, per_cta = kGW * warps, lines = FAM == 3 ? a.k.H : a.k.W;
+template <int CPL, bool S8, int FAM, bool BANDED, bool ADD = false>
+static cudaError_t launch_family(const LineArgs &a, int nf, int dirs, bool overlap, cudaStream_t s) {
+  constexpr int kWarp = kLineAhead * 32 * CPL * (ADD ? 3 : 1) + (BANDED ? kGW * kGL * CPL * 2 : 0);
+  constexpr int kFit = 224 * 1024 / kWarp, kMaxWarps = kFit < 8 ? kFit : 8;   // (the ADD walks' rings are three times as long)
+  const int warps = std::min(a.k.line_warps, kMaxWarps), per_cta = kGW * warps, lines = FAM == 3 ? a.k.H : a.k.W;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((lines + per_cta - 1) / per_cta, 2, nf);
+  cfg.gridDim = dim3((lines + per_cta - 1) / per_cta, dirs, nf);
   cfg.blockDim = dim3(32 * warps);
-  cfg.dynamicSmemBytes = warps * kLineAhead * 32 * CPL;
+  cfg.dynamicSmemBytes = warps * kWarp;
   static bool done[64] = {};
-  const cudaError_t e = smem_optin(k_lines<CPL, S8, FAM>, 8 * kLineAhead * 32 * CPL, done);
+  const cudaError_t e = smem_optin(k_lines<CPL, S8, FAM, BANDED, ADD>, kMaxWarps * kWarp, done);
   if (e != cudaSuccess) return e;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -179,13 +223,13 @@ static cudaError_t launch_family(const LineArgs &a, int nf, bool overlap, cudaSt
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = overlap ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k_lines<CPL, S8, FAM>, a);
+  return cudaLaunchKernelEx(&cfg, k_lines<CPL, S8, FAM, BANDED, ADD>, a);
 }
 
 // Where a family's down and up vectors of a pixel lie.  S8: side by side,
 // [down Dp bytes][up Dp bytes], in the family's buffer (rows: in the fourth
 // spill region); u16: the up vectors in the family's buffer, the down vectors
-// in the family's spill region.
+// in the family's spill region, the rows' one sum in the fourth.
 inline void family_vectors(const KParams &k, const Buffers &b, bool s8, int fam, uint8_t *(&v)[2], size_t (&frame)[2]) {
   const size_t cells = frame_cells(k);
   uint8_t *region = static_cast<uint8_t *>(b.spill) + fam * 2 * cells;
@@ -196,37 +240,56 @@ inline void family_vectors(const KParams &k, const Buffers &b, bool s8, int fam,
     frame[0] = frame[1] = (fam < 3 ? 2 : 8) * cells;
   } else {
     v[0] = region;
-    v[1] = part;
+    v[1] = fam < 3 ? part : region;
     frame[0] = 8 * cells;
-    frame[1] = 2 * cells;
+    frame[1] = (fam < 3 ? 2 : 8) * cells;
   }
 }
 
-template <int CPL, bool S8>
-cudaError_t launch_lines_t(const KParams &k, const Buffers &b, int nf, cudaStream_t s) {
-  LineArgs a;
+template <int CPL, bool S8, bool BANDED>
+static cudaError_t launch_walks(const KParams &k, const Buffers &b, int nf, cudaStream_t s) {
+  LineArgs a = {};
   a.k = k;
+  if (BANDED) a.k.D = k.Dp;                      // cells are band positions
   a.cost = b.cost;
   a.sc.p1x2 = (uint32_t)k.p1 * 0x10001u;
   a.sc.dpx2 = (uint32_t)(k.p2 - k.p1) * 0x10001u;
   a.gate = b.gate;
+  a.lo = b.band_lo;
   // the first launch waits for the cost volume as usual; the others may start
   // beside it (they touch nothing it writes).  The rows, the longest walks, go
-  // first; only byte vectors: the row kernel walks the rows of u16 costs
+  // first; with u16 costs their second direction adds to the first one's
+  // vectors: two launches, the second after everything before it
   bool overlap = false;
+  cudaError_t e = cudaSuccess;
   auto family = [&](auto fam) {
     constexpr int F = decltype(fam)::value;
+    if (e != cudaSuccess) return;
     family_vectors(k, b, S8, F, a.dst, a.dst_frame);
-    const cudaError_t e = launch_family<CPL, S8, F>(a, nf, overlap, s);
+    if constexpr (F == 3 && !S8) {
+      a.dir = 0;
+      e = launch_family<CPL, S8, F, BANDED>(a, nf, 1, false, s);
+      a.dir = 1;
+      if (e == cudaSuccess) e = launch_family<CPL, S8, F, BANDED, true>(a, nf, 1, false, s);
+    } else {
+      e = launch_family<CPL, S8, F, BANDED>(a, nf, 2, overlap, s);
+    }
     overlap = true;
-    return e;
   };
-  cudaError_t e = cudaSuccess;
-  if constexpr (S8) e = family(std::integral_constant<int, 3>{});
-  if (e == cudaSuccess) e = family(std::integral_constant<int, 0>{});
-  if (e == cudaSuccess && k.num_paths == 8) e = family(std::integral_constant<int, 1>{});
-  if (e == cudaSuccess && k.num_paths == 8) e = family(std::integral_constant<int, 2>{});
+  family(std::integral_constant<int, 3>{});
+  family(std::integral_constant<int, 0>{});
+  if (k.num_paths == 8) {
+    family(std::integral_constant<int, 1>{});
+    family(std::integral_constant<int, 2>{});
+  }
   return e;
+}
+
+template <int CPL, bool S8>
+cudaError_t launch_lines_t(const KParams &k, const Buffers &b, int nf, cudaStream_t s) {
+  if constexpr (CPL <= 16)
+    if (k.band) return launch_walks<CPL, S8, true>(k, b, nf, s);
+  return launch_walks<CPL, S8, false>(k, b, nf, s);
 }
 
 }  // namespace oct

@@ -1,4 +1,4 @@
-// sgmf_rows.cuh -- the two horizontal directions of Eq. 2, the path sum S, the
+// sgmf_rows.cuh -- behind the sweep: the two horizontal directions of Eq. 2, the path sum S, the
 // winner d* (Eq. 3) and the right view's d' (Sec. IV-C).
 //
 // A CTA takes four image rows: its first warp walks them left -> right
@@ -27,7 +27,7 @@
 namespace sgmf {
 namespace oct {
 
-constexpr int kMaxVec = 6;      // vectors read per pixel beside cost and spill
+constexpr int kMaxVec = 2;      // u16 vectors (the sweep's sums) read per pixel beside cost and spill
 
 struct RowArgs {
   KParams k;
@@ -72,7 +72,7 @@ struct RowLane {
   bool act;                     // the group's row is inside the image
   size_t row;                   // its first pixel
   uint32_t z[CPL / 4], kb[CPL / 2];
-  uint32_t lo_edge, hi_edge;
+  Edges edges;
   int end_lane, end_cell;       // where disparity D - 1 lies
   StepConsts sc;
   uint8_t *spill;               // the lane's first chunk of the row's spill
@@ -89,7 +89,7 @@ __device__ __forceinline__ void row_step(RowWalk<CPL> &w, const RowLane<CPL> &g,
   const uint32_t z0[CPL / 4] = {};
   uint32_t C[NW];
   slot8<CPL>(slot, g.lane, g.z, C);
-  step<NW>(w.L, C, w.mm, g.sc, g.lo_edge, g.hi_edge);
+  step<NW>(w.L, C, w.mm, g.sc, g.edges);
   w.mm = group_min<NW>(w.L);
   if constexpr (!SECOND) {
     if (g.act) VecW<CPL, S8>::put(g.spill + (size_t)x * Dp * CF::SB, w.L);
@@ -274,8 +274,7 @@ __global__ void __launch_bounds__(64) k_rows(const __grid_constant__ RowArgs a) 
     g.kb[i] = (uint32_t)(d0 & 0xff) | ((uint32_t)(d1 & 0xff) << 8) | (d0 >= D ? 0xff0000u : 0u) |
               (d1 >= D ? 0xff000000u : 0u);
   }
-  g.lo_edge = lig == 0 ? 0xffffu : 0u;
-  g.hi_edge = lig == kGL - 1 ? 0xffff0000u : 0u;
+  g.edges = no_neighbours(lig);
   g.end_lane = (D - 1) / CPL;
   g.end_cell = (D - 1) % CPL;
   g.sc = a.sc;
@@ -332,20 +331,11 @@ cudaError_t launch_rows_t(const KParams &k, const Buffers &b, int nf, cudaStream
   a.sc.p1x2 = (uint32_t)k.p1 * 0x10001u;
   a.sc.dpx2 = (uint32_t)(k.p2 - k.p1) * 0x10001u;
   a.gate = b.gate;
-  // the sweep's two sums, or the line families' up vectors, then their down ones
-  const int nfam = k.sweep ? 2 : (k.num_paths == 8 ? 3 : 1);
-  for (int i = 0; i < nfam; ++i) {
+  for (int i = 0; i < 2; ++i) {
     a.vec[i] = reinterpret_cast<const uint8_t *>(b.part[i]);
     a.vec_frame[i] = 2 * cells;
-    if (!k.sweep) {
-      a.vec[nfam + i] = static_cast<const uint8_t *>(b.spill) + i * 2 * cells;
-      a.vec_frame[nfam + i] = 8 * cells;
-    }
   }
-  if (k.sweep) return launch_rows_v<CPL, S8, 2>(a, nf, s);
-  if constexpr (!S8)
-    return k.num_paths == 8 ? launch_rows_v<CPL, S8, 6>(a, nf, s) : launch_rows_v<CPL, S8, 2>(a, nf, s);
-  return cudaErrorInvalidValue;   // byte vectors of the line kernels: launch_wta_t
+  return launch_rows_v<CPL, S8, 2>(a, nf, s);
 }
 
 }  // namespace oct

@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(32 * SweepCfg<CPL>::kMaxWarps, 1) k_sweep(cons
 
   uint32_t z[CPL / 4];
   pad_bytes<CPL>(a.k.D, lig, z);
-  const uint32_t lo_edge = lig == 0 ? 0xffffu : 0u, hi_edge = lig == kGL - 1 ? 0xffff0000u : 0u;
+  const Edges none = no_neighbours(lig);
   const StepConsts sc = a.sc;
   // path-cost vectors of the group's pixels and their minima: vertical,
   // from-left diagonal (predecessor x - 1), from-right diagonal (x + 1)
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(32 * SweepCfg<CPL>::kMaxWarps, 1) k_sweep(cons
   // one Eq. 2 step from predecessor (pr, mp) on costs Cc: the new vector and its min
   auto move = [&](uint32_t(&o)[NW], uint32_t &mo, const uint32_t(&pr)[NW], uint32_t mp, const uint32_t(&Cc)[NW]) {
     copy_vec<NW>(o, pr);
-    step<NW>(o, Cc, mp, sc, lo_edge, hi_edge);
+    step<NW>(o, Cc, mp, sc, none);
     mo = group_min<NW>(o);
   };
   bool ok = true;
@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(32 * SweepCfg<CPL>::kMaxWarps, 1) k_sweep(cons
       uint32_t sum[NW];
 #pragma unroll
       for (int w = 0; w < NW; ++w) sum[w] = V[i][w] + DL[i][w] + DR[i][w];
-      const int x = xg + i;
+      [[maybe_unused]] const int x = xg + i;
       if constexpr (CF::kBulkSums)   // into the row's staging buffer (pixels outside the image are not copied out)
         store_u16<CPL>(wsum + (t & 1) * CF::kSumBuf + (grp * P + i) * Dp * 2 + lig * Vec16<CPL>::kLane, sum);
       else if (ok && x < W)
@@ -486,15 +486,16 @@ cudaError_t launch_sweep_t(const KParams &k, const Buffers &b, int nf, cudaStrea
 }  // namespace sgmf
 
 // explicit instantiations of one lane width (CPL cells per lane)
-#define SGMF_OCT_INSTANTIATE(CPL)                                                                       \
-  namespace sgmf {                                                                                      \
-  namespace oct {                                                                                       \
-  template cudaError_t launch_lines_t<CPL, false>(const KParams &, const Buffers &, int, cudaStream_t); \
-  template cudaError_t launch_lines_t<CPL, true>(const KParams &, const Buffers &, int, cudaStream_t);  \
-  template cudaError_t launch_rows_t<CPL, false>(const KParams &, const Buffers &, int, cudaStream_t);  \
-  template cudaError_t launch_rows_t<CPL, true>(const KParams &, const Buffers &, int, cudaStream_t);   \
-  template cudaError_t launch_sweep_t<CPL>(const KParams &, const Buffers &, int, cudaStream_t);        \
-  template int sweep_plan_t<CPL>(const KParams &, int, int *);                                          \
-  template cudaError_t launch_wta_t<CPL>(const KParams &, const Buffers &, int, int16_t *, cudaStream_t); \
-  }                                                                                                     \
+#define SGMF_AGG_INSTANTIATE(CPL)                                                                              \
+  namespace sgmf {                                                                                             \
+  namespace oct {                                                                                              \
+  template cudaError_t launch_lines_t<CPL, false>(const KParams &, const Buffers &, int, cudaStream_t);        \
+  template cudaError_t launch_lines_t<CPL, true>(const KParams &, const Buffers &, int, cudaStream_t);         \
+  template cudaError_t launch_rows_t<CPL, false>(const KParams &, const Buffers &, int, cudaStream_t);         \
+  template cudaError_t launch_rows_t<CPL, true>(const KParams &, const Buffers &, int, cudaStream_t);          \
+  template cudaError_t launch_wta_t<CPL, false>(const KParams &, const Buffers &, int, int16_t *, cudaStream_t); \
+  template cudaError_t launch_wta_t<CPL, true>(const KParams &, const Buffers &, int, int16_t *, cudaStream_t); \
+  template cudaError_t launch_sweep_t<CPL>(const KParams &, const Buffers &, int, cudaStream_t);               \
+  template int sweep_plan_t<CPL>(const KParams &, int, int *);                                                 \
+  }                                                                                                            \
   }

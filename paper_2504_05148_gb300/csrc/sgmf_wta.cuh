@@ -1,21 +1,24 @@
 // sgmf_wta.cuh -- path sum S, winner d* (Eq. 3), the right view's d' and the
-// three-view check (Eq. 6) from the line walks' byte vectors.
+// three-view check (Eq. 6) from vectors of path costs in memory.
 //
-// Where every direction's path costs lie in memory as byte vectors (line
-// kernels, costs that fit a byte), nothing is left to walk: a CTA takes one
-// image row, each of its 8-lane groups a segment of it, so that a call of few
-// frames fills the GPU.  The kernel is bound by reading the vectors (8 bytes a
-// cell with eight paths), which its lanes copy ahead into their places of a
-// shared-memory ring (cp.async).  Measured on 1242 x 375, D = 128: 113 us for
-// one frame, 605 us for 8 (6.3 TB/s), check included, where the row walk that
-// formed S on the way and the check kernel took 371 and 985 us.
+// Behind the line walks every direction's path costs lie in memory and nothing
+// is left to walk: a CTA takes one image row, each of its 8-lane groups a
+// segment of it, so that a call of few frames fills the GPU.  The kernel is
+// bound by reading the vectors (8 bytes a cell with eight directions' byte
+// vectors), which its lanes copy ahead into their places of a shared-memory
+// ring (cp.async).  Measured on 1242 x 375, D = 128: 113 us for one frame,
+// 605 us for 8 (6.3 TB/s), check included, where the row walk that formed S on
+// the way and the check kernel took 371 and 985 us.
 //
 // d' is a systolic running min inside a segment: the best key S << 8 | d of
 // right pixel x' = x - d moves one disparity slot per step; the slot that
 // leaves, and at the segment's end the slots left, are min-merged into the
-// row's d' keys in shared memory.  Then the row's check: every pixel's stereo
-// term from those keys, and the LiDAR term, gathered over the row, for the
-// pixels it decides.
+// row's d' keys in shared memory.  On the bands the slots are band positions
+// (slot s: right pixel x - lo - s) and all leave where the band start changes;
+// segments are whole band tiles, so that this is every eighth step for the four
+// groups of a warp together.  Then the row's check: every pixel's stereo term
+// from those keys, and the LiDAR term, gathered over the row, for the pixels it
+// decides.
 #pragma once
 
 #include "sgmf_check.cuh"
@@ -24,30 +27,35 @@
 namespace sgmf {
 namespace oct {
 
+constexpr int kMaxWtaVec = 7;
+
 struct WtaArgs {
   KParams k;
   Buffers b;                    // frame 0's maps (d*, d', d-sub, row ORs, gate)
-  const uint8_t *vec[4];        // frame 0's vector pairs: two byte vectors, 2 Dp bytes per pixel
-  size_t vec_frame[4];          // bytes from one frame to the next
+  const uint8_t *vec[kMaxWtaVec];   // frame 0's vectors, 2 Dp bytes per pixel
+  size_t vec_frame[kMaxWtaVec];     // bytes from one frame to the next
   uint16_t *dbg_sum;            // frame 0's S (u16 vectors), or null
   int16_t *out;
 };
 
-// NP: vector pairs
-template <int CPL, int NP>
+// NP: pairs of byte vectors side by side; NS: u16 vectors (after the pairs)
+template <int CPL, int NP, int NS>
 struct WtaCfg {
-  static constexpr int Dp = kGL * CPL, kVec = 32 * CPL, kSlot = 2 * NP * kVec;
-  static constexpr int R = CPL == 8 ? 8 : (CPL == 16 ? 4 : 2);   // slots: one step each, about 16 KB a warp
-  static constexpr int kMaxWarps = 8;
+  static constexpr int Dp = kGL * CPL, k8 = 32 * CPL, NV = NP + NS, kSlot = 2 * NV * k8;
+  // slots: one step each, about 16 KB a warp (at least 2)
+  static constexpr int R = kSlot * 8 <= 16384 ? 8 : (kSlot * 4 <= 16384 ? 4 : 2);
+  // at most 8 warps a CTA, and what the shared memory of the widest row leaves
+  static constexpr int kFit = (226 * 1024 - kMaxDim * 8) / (R * kSlot), kMaxWarps = kFit < 8 ? kFit : 8;
+  static_assert(kMaxWarps >= 1, "a warp's ring fits beside the widest row");
   static int warps(int W) { return max(1, min(kMaxWarps, (W + 319) / 320)); }   // segments of about 80 pixels
   // the rings, the row's d' keys (u32), d* and the list of undecided pixels (u16)
   static int smem(int W) { return warps(W) * R * kSlot + (W + 3) / 4 * 4 * 8; }
 };
 
-template <int CPL, int NP>
+template <int CPL, int NP, int NS, bool BANDED>
 __global__ void __launch_bounds__(256) k_wta(const __grid_constant__ WtaArgs a) {
-  using CF = WtaCfg<CPL, NP>;
-  constexpr int NW = CPL / 2, Dp = CF::Dp, R = CF::R;
+  using CF = WtaCfg<CPL, NP, NS>;
+  constexpr int NW = CPL / 2, Dp = CF::Dp, R = CF::R, NV = CF::NV;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ int n_list;
   const int f = blockIdx.y, y = blockIdx.x;
@@ -65,19 +73,27 @@ __global__ void __launch_bounds__(256) k_wta(const __grid_constant__ WtaArgs a) 
   __syncthreads();
   {
     // the group's segment [x0, x1): equal lengths, the last ones may be short or empty
-    const int seg = (W + kGW * nwarp - 1) / (kGW * nwarp), gi = warp * kGW + grp;
+    int seg = (W + kGW * nwarp - 1) / (kGW * nwarp);
+    if constexpr (BANDED) seg = (seg + kBandTile - 1) / kBandTile * kBandTile;
+    const int gi = warp * kGW + grp;
     const int x0 = min(gi * seg, W), x1 = min(x0 + seg, W);
     uint8_t *ring = smem + warp * R * CF::kSlot;
     const uint32_t ring_s = smem_u32(ring);
-    const uint8_t *pv[NP];
+    const uint8_t *pv[NV];
 #pragma unroll
-    for (int j = 0; j < NP; ++j)
-      pv[j] = a.vec[j] + f * a.vec_frame[j] + (row + min(x0, W - 1)) * 2 * Dp + lig * Vec8<CPL>::kLane;
+    for (int j = 0; j < NV; ++j)
+      pv[j] = a.vec[j] + f * a.vec_frame[j] + (row + min(x0, W - 1)) * 2 * Dp +
+              lig * (j < NP ? Vec8<CPL>::kLane : Vec16<CPL>::kLane);
     auto copy = [&](uint32_t slot, bool move) {
 #pragma unroll
-      for (int j = 0; j < NP; ++j) {
-        copy8<CPL>(slot + 2 * j * CF::kVec, lane, pv[j]);
-        copy8<CPL>(slot + (2 * j + 1) * CF::kVec, lane, pv[j] + Dp);
+      for (int j = 0; j < NV; ++j) {
+        const uint32_t d = slot + 2 * j * CF::k8;
+        if (j < NP) {
+          copy8<CPL>(d, lane, pv[j]);
+          copy8<CPL>(d + CF::k8, lane, pv[j] + Dp);
+        } else {
+          copy16<CPL>(d, lane, pv[j]);
+        }
         if (move) pv[j] += 2 * Dp;
       }
     };
@@ -86,14 +102,20 @@ __global__ void __launch_bounds__(256) k_wta(const __grid_constant__ WtaArgs a) 
       copy(ring_s + t * CF::kSlot, x0 + t + 1 < x1);
       cp_commit();
     }
-    uint32_t kb[NW];
+    uint32_t kb[NW];                             // the keys' low bytes (d) and the padding's high ones
+    [[maybe_unused]] const int16_t *lo_row = nullptr;
+    [[maybe_unused]] int lo = 0;                 // the band start of the tile
+    if constexpr (BANDED) {
+      lo_row = b.band_lo + (y >> kBandTileLog) * a.k.tw;
+    } else {
 #pragma unroll
-    for (int i = 0; i < NW; ++i) {
-      const int d0 = lig * CPL + i, d1 = d0 + NW;
-      kb[i] = (uint32_t)(d0 & 0xff) | ((uint32_t)(d1 & 0xff) << 8) | (d0 >= D ? 0xff0000u : 0u) |
-              (d1 >= D ? 0xff000000u : 0u);
+      for (int i = 0; i < NW; ++i) {
+        const int d0 = lig * CPL + i, d1 = d0 + NW;
+        kb[i] = (uint32_t)(d0 & 0xff) | ((uint32_t)(d1 & 0xff) << 8) | (d0 >= D ? 0xff0000u : 0u) |
+                (d1 >= D ? 0xff000000u : 0u);
+      }
     }
-    const int end_lane = (D - 1) / CPL, end_cell = (D - 1) % CPL;
+    const int end_lane = BANDED ? kGL - 1 : (D - 1) / CPL, end_cell = BANDED ? CPL - 1 : (D - 1) % CPL;
     uint8_t *dbg = (f == 0 && a.dbg_sum != nullptr)
                        ? reinterpret_cast<uint8_t *>(a.dbg_sum) + row * Dp * 2 + lig * Vec16<CPL>::kLane
                        : nullptr;
@@ -101,21 +123,52 @@ __global__ void __launch_bounds__(256) k_wta(const __grid_constant__ WtaArgs a) 
 #pragma unroll
     for (int j = 0; j < CPL; ++j) acc[j] = 0xffffffffu;
     const uint32_t z0[CPL / 4] = {};
+    // every slot of the accumulator to the row's keys; x: the pixel they were last updated at
+    auto flush = [&](int x) {
+#pragma unroll
+      for (int j = 0; j < CPL; ++j) {
+        const int xr = x - lo - (lig * CPL + j);
+        if ((BANDED ? acc[j] != 0xffffffffu : lig * CPL + j < D) && xr >= 0) atomicMin(&merge[xr], acc[j]);
+      }
+    };
     int base = 0;
     for (int t = 0; t < seg; ++t) {
       const int x = x0 + t;
       const bool act = x < x1;
+      if constexpr (BANDED) {
+        if (t % kBandTile == 0) {
+          const int now = lo_row[min(x, W - 1) >> kBandTileLog];
+          if (t == 0 || now != lo) {
+            if (t > 0 && act) flush(x - 1);      // (a group past its end was flushed there)
+#pragma unroll
+            for (int j = 0; j < CPL; ++j) acc[j] = 0xffffffffu;
+            lo = now;
+            const uint32_t b0 = (uint32_t)(lo + lig * CPL);
+#pragma unroll
+            for (int i = 0; i < NW; ++i) kb[i] = (b0 + i) | ((b0 + i + NW) << 8);
+          }
+          __syncwarp();
+        }
+      }
       cp_wait<R - 1>();
       uint32_t Sm[NW];
 #pragma unroll
       for (int w = 0; w < NW; ++w) Sm[w] = 0u;
 #pragma unroll
-      for (int j = 0; j < NP; ++j) {
-        uint32_t T[NW], U[NW];
-        slot8<CPL>(ring + base + 2 * j * CF::kVec, lane, z0, T);
-        slot8<CPL>(ring + base + (2 * j + 1) * CF::kVec, lane, z0, U);
+      for (int j = 0; j < NV; ++j) {
+        const uint8_t *v = ring + base + 2 * j * CF::k8;
+        uint32_t T[NW];
+        if (j < NP) {
+          uint32_t U[NW];
+          slot8<CPL>(v, lane, z0, T);
+          slot8<CPL>(v + CF::k8, lane, z0, U);
 #pragma unroll
-        for (int i = 0; i < NW; ++i) Sm[i] = j == 0 ? T[i] + U[i] : Sm[i] + T[i] + U[i];
+          for (int i = 0; i < NW; ++i) Sm[i] = j == 0 ? T[i] + U[i] : Sm[i] + T[i] + U[i];
+        } else {
+          slot16<CPL>(v, lane, T);
+#pragma unroll
+          for (int i = 0; i < NW; ++i) Sm[i] = j == 0 ? T[i] : Sm[i] + T[i];
+        }
       }
       copy(ring_s + base, x + R + 1 < x1);
       cp_commit();
@@ -141,7 +194,7 @@ __global__ void __launch_bounds__(256) k_wta(const __grid_constant__ WtaArgs a) 
         ds_s[x] = (uint16_t)ds;
         b.dstar[row + x] = (int16_t)ds;
       }
-      if (a.k.subpixel) {
+      if (!BANDED && a.k.subpixel) {
         // parabola through S(d*-1), S(d*), S(d*+1); the lanes holding the two
         // neighbours contribute them, every other lane the neutral 0xffffffff
         uint32_t sm = 0xffffffffu, sp = 0xffffffffu;
@@ -161,10 +214,10 @@ __global__ void __launch_bounds__(256) k_wta(const __grid_constant__ WtaArgs a) 
       for (int j = CPL - 1; j > 0; --j) acc[j] = min(acc[j - 1], key[j]);
       acc[0] = min(lig == 0 ? 0xffffffffu : below, key[0]);
       if (act && t + 1 < x1 - x0) {
-        const int xr = x - (D - 1);              // slot D - 1 leaves
+        const int xr = x - lo - (BANDED ? Dp - 1 : D - 1);   // the last slot leaves
         if (lig == end_lane && xr >= 0) {
           uint32_t v = acc[CPL - 1];
-          if (end_cell != CPL - 1) {
+          if (!BANDED && end_cell != CPL - 1) {
 #pragma unroll
             for (int j = 0; j < CPL - 1; ++j)
               if (j == end_cell) v = acc[j];
@@ -172,12 +225,7 @@ __global__ void __launch_bounds__(256) k_wta(const __grid_constant__ WtaArgs a) 
           atomicMin(&merge[xr], v);
         }
       } else if (act) {
-        // the segment's last pixel: every slot leaves
-#pragma unroll
-        for (int j = 0; j < CPL; ++j) {
-          const int d = lig * CPL + j;
-          if (d < D && x >= d) atomicMin(&merge[x - d], acc[j]);
-        }
+        flush(x);                                // the segment's last pixel: every slot leaves
       }
     }
     cp_wait<0>();
@@ -186,8 +234,14 @@ __global__ void __launch_bounds__(256) k_wta(const __grid_constant__ WtaArgs a) 
   // the row's d' and the stereo term; the pixels left to the LiDAR term are listed
   for (int x = threadIdx.x; x < W; x += blockDim.x) {
     const int ds = ds_s[x], xm = x - ds;
-    b.dprime[row + x] = (int16_t)(merge[x] & 0xffu);
-    const bool stereo = xm >= 0 && abs(ds - (int)(merge[xm] & 0xffu)) <= a.k.lr;
+    // (on the bands a right pixel whose diagonal meets no band has none: -1,
+    // and the stereo term fails)
+    b.dprime[row + x] = BANDED && merge[x] == 0xffffffffu ? (int16_t)-1 : (int16_t)(merge[x] & 0xffu);
+    bool stereo = false;
+    if (xm >= 0) {
+      const uint32_t m = merge[xm];
+      stereo = (!BANDED || m != 0xffffffffu) && abs(ds - (int)(m & 0xffu)) <= a.k.lr;
+    }
     if (check_needs_lidar(a.k, stereo))
       list[atomicAdd(&n_list, 1)] = (uint16_t)x;
     else
@@ -200,33 +254,50 @@ __global__ void __launch_bounds__(256) k_wta(const __grid_constant__ WtaArgs a) 
   }
 }
 
-template <int CPL, int NP>
+template <int CPL, int NP, int NS, bool BANDED>
 static cudaError_t launch_wta_v(const WtaArgs &a, int nf, cudaStream_t s) {
-  using CF = WtaCfg<CPL, NP>;
+  using CF = WtaCfg<CPL, NP, NS>;
   static bool done[64] = {};
   const int most = CF::kMaxWarps * CF::R * CF::kSlot + kMaxDim * 8;
-  cudaError_t e = smem_optin(k_wta<CPL, NP>, most, done);
+  cudaError_t e = smem_optin(k_wta<CPL, NP, NS, BANDED>, most, done);
   if (e != cudaSuccess) return e;
-  k_wta<CPL, NP><<<dim3(a.k.H, nf), 32 * CF::warps(a.k.W), CF::smem(a.k.W), s>>>(a);
+  k_wta<CPL, NP, NS, BANDED><<<dim3(a.k.H, nf), 32 * CF::warps(a.k.W), CF::smem(a.k.W), s>>>(a);
   return cudaGetLastError();
 }
 
-template <int CPL>
-cudaError_t launch_wta_t(const KParams &k, const Buffers &b, int nf, int16_t *out, cudaStream_t s) {
+template <int CPL, bool S8, bool BANDED>
+static cudaError_t launch_wta_b(const KParams &k, const Buffers &b, int nf, int16_t *out, cudaStream_t s) {
   WtaArgs a = {};
   a.k = k;
   a.b = b;
   a.dbg_sum = b.dbg_sum;
   a.out = out;
+  int n = 0;
+  auto add = [&](const uint8_t *v, size_t frame) {
+    a.vec[n] = v;
+    a.vec_frame[n++] = frame;
+  };
   const int nfam = k.num_paths == 8 ? 3 : 1;
-  for (int i = 0; i <= nfam; ++i) {
-    uint8_t *v[2];
-    size_t frame[2];
-    family_vectors(k, b, true, i == nfam ? 3 : i, v, frame);
-    a.vec[i] = v[0];
-    a.vec_frame[i] = frame[0];
+  uint8_t *v[2];
+  size_t frame[2];
+  family_vectors(k, b, S8, 3, v, frame);
+  add(v[0], frame[0]);                           // the rows: a pair of byte vectors, or their u16 sum
+  for (int i = 0; i < nfam; ++i) {
+    family_vectors(k, b, S8, i, v, frame);
+    add(v[0], frame[0]);
+    if (!S8) add(v[1], frame[1]);
   }
-  return nfam == 3 ? launch_wta_v<CPL, 4>(a, nf, s) : launch_wta_v<CPL, 2>(a, nf, s);
+  if constexpr (S8)
+    return nfam == 3 ? launch_wta_v<CPL, 4, 0, BANDED>(a, nf, s) : launch_wta_v<CPL, 2, 0, BANDED>(a, nf, s);
+  else
+    return nfam == 3 ? launch_wta_v<CPL, 0, 7, BANDED>(a, nf, s) : launch_wta_v<CPL, 0, 3, BANDED>(a, nf, s);
+}
+
+template <int CPL, bool S8>
+cudaError_t launch_wta_t(const KParams &k, const Buffers &b, int nf, int16_t *out, cudaStream_t s) {
+  if constexpr (CPL <= 16)
+    if (k.band) return launch_wta_b<CPL, S8, true>(k, b, nf, out, s);
+  return launch_wta_b<CPL, S8, false>(k, b, nf, out, s);
 }
 
 }  // namespace oct
