@@ -551,6 +551,21 @@ static sgmf_status finish(sgmf_ctx *c, const KParams &ka, const Buffers &b, int 
   return SGMF_OK;
 }
 
+// Whether the line walks of a call of n frames store the vectors of every
+// second row (column) only and the winner kernel takes the others' steps: 17
+// instead of 24 bytes a cell through memory for about half as many instructions
+// again in the winner kernel.  It pays where the volumes are far larger than the
+// L2 (1242 x 375, D = 128: one frame of 60 M cells 377 -> 397 us, two 651 -> 616,
+// eight 2100 -> 1943; four paths, half the walks to save on: 119 M cells 416 ->
+// 425, 238 M 646 -> 628) and where a lane's 16 or 24 cells spread the steps'
+// fixed work without filling the registers: at Dp = 64 640 x 480 x 12 1411 ->
+// 1504 us, at Dp = 256 1920 x 1080 x 4 8550 -> 10460.
+static int half_vectors(const sgmf_ctx *c, int n) {
+  const KParams &k = c->k;
+  return c->spill8 && !k.band && (k.Dp == 128 || k.Dp == 192) &&
+         frame_cells(k) * n >= (k.num_paths == 8 ? 100000000u : 200000000u);
+}
+
 // Aggregation, winners and check of the n frames whose cost volume is made.
 // A sweep batch goes through in parts of m frames: part i's sweep on the
 // context's stream, then the rest of it on the side stream while part i + 1 is
@@ -559,7 +574,8 @@ static sgmf_status finish(sgmf_ctx *c, const KParams &ka, const Buffers &b, int 
 // sweep was measured twice and gave nothing: 8.17-8.24 against 8.20 ms for 32
 // KITTI frames, and 3 % slower at 64; the sweep slows by what they save.)
 static sgmf_status aggregate(sgmf_ctx *c, int n, int16_t *out, cudaStream_t s) {
-  const KParams ka = agg_params(c);
+  KParams ka = agg_params(c);
+  ka.half = half_vectors(c, n);
   const int m = ka.sweep ? sweep_part(c, n) : 0;
   if (m == 0) {
     if (ka.sweep) TIMED(c, "agg_sweep", s, launch_agg_sweep(ka, c->b, n, s));

@@ -227,7 +227,16 @@ __device__ __forceinline__ void pad_bytes(int D, int lig, uint32_t (&z)[CPL / 4]
 struct StepConsts {
   uint32_t p1x2;   // P1 in both halves
   uint32_t dpx2;   // (P2 - P1) in both halves
+  uint32_t one;    // 1, as a value the compiler cannot see
 };
+inline StepConsts step_consts(const KParams &k) {
+  return {(uint32_t)k.p1 * 0x10001u, (uint32_t)(k.p2 - k.p1) * 0x10001u, 1u};
+}
+__device__ __forceinline__ uint32_t mad_u32(uint32_t a, uint32_t b, uint32_t c) {
+  uint32_t d;
+  asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+  return d;
+}
 
 // The group's outer neighbours, as bits ORed into the first / last lane's words:
 // 0xffff in the missing neighbour's half (L(-1), L(Dp) only enter a min).  On the
@@ -241,7 +250,11 @@ __device__ __forceinline__ Edges no_neighbours(int lig) {
 }
 
 // One step of Eq. 2 for the lane's words.  mm = min_k L(p - r, k) in both halves.
-template <int NW, bool BANDED = false>
+// MAD: the last addition as a multiply-add (t * 1 + ..), which leaves the ALU
+// pipe, the bound of most callers, for the FMA pipe: 2 to 4 % of the walks and
+// the winner kernel at up to 8 words a lane; above, and in the sweep at 8, the
+// register it costs loses more.
+template <int NW, bool BANDED = false, bool MAD = NW <= 8>
 __device__ __forceinline__ void step(uint32_t (&L)[NW], const uint32_t (&C)[NW], uint32_t mm, const StepConsts &sc,
                                      Edges e, int lig = 0) {
   const uint32_t below = __shfl_up_sync(kAll, L[NW - 1], 1, kGL);
@@ -262,7 +275,7 @@ __device__ __forceinline__ void step(uint32_t (&L)[NW], const uint32_t (&C)[NW],
     const uint32_t right = i == NW - 1 ? last : L[i + 1];
     const uint32_t t = __viaddmin_u16x2(__vimin3_u16x2(left, right, cap), sc.p1x2, L[i]);
     left = L[i];
-    L[i] = t + C[i] + negmm;
+    L[i] = MAD ? mad_u32(t, sc.one, C[i] + negmm) : t + C[i] + negmm;
   }
 }
 
@@ -290,6 +303,19 @@ __device__ __forceinline__ uint32_t group_min(const uint32_t (&L)[NW]) {
   const uint32_t a = __shfl_xor_sync(kAll, v, 1), b = __shfl_xor_sync(kAll, v, 2), c = __shfl_xor_sync(kAll, v, 3);
   v = __vminu2(__vimin3_u16x2(v, a, b), c);
   return __vminu2(v, __shfl_xor_sync(kAll, v, 4));
+}
+
+// the minima of two vectors, each in both halves: one pass of shuffles for both
+template <int NW>
+__device__ __forceinline__ void group_min2(const uint32_t (&A)[NW], const uint32_t (&B)[NW], uint32_t &ma,
+                                           uint32_t &mb) {
+  const uint32_t va = lane_min<NW>(A), vb = lane_min<NW>(B);
+  uint32_t v = __vminu2(prmt(va, vb, 0x5410), prmt(va, vb, 0x7632));
+  const uint32_t a = __shfl_xor_sync(kAll, v, 1), b = __shfl_xor_sync(kAll, v, 2), c = __shfl_xor_sync(kAll, v, 3);
+  v = __vminu2(__vimin3_u16x2(v, a, b), c);
+  v = __vminu2(v, __shfl_xor_sync(kAll, v, 4));
+  ma = prmt(v, v, 0x1010);
+  mb = prmt(v, v, 0x3232);
 }
 
 // min of a u32 over the group

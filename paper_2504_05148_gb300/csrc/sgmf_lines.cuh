@@ -62,9 +62,11 @@ struct LinePos {
 
 constexpr int kLineAhead = 16;   // steps copied ahead (a multiple of the four unrolled)
 
+// HALF: store only the vectors of even rows (rows family: even columns); the
+// winner kernel takes the others' step itself.
 // ADD: the vector of the pixel's other direction, there already, is added (u16
 // rows: one vector for both).  BANDED: on the bands (no padding cells).
-template <int CPL, bool S8, int FAM, bool BANDED, bool ADD>
+template <int CPL, bool S8, int FAM, bool BANDED, bool ADD, bool HALF>
 __global__ void __launch_bounds__(256) k_lines(const __grid_constant__ LineArgs a) {
   constexpr int NW = CPL / 2, Dp = kGL * CPL, A = kLineAhead, U = 4, k8 = 32 * CPL, kSlot = k8 * (ADD ? 3 : 1);
   static_assert(!(ADD && S8), "byte vectors have a place each");
@@ -175,7 +177,7 @@ __global__ void __launch_bounds__(256) k_lines(const __grid_constant__ LineArgs 
 #pragma unroll
       for (int w = 0; w < NW; ++w) other[w] += L[w];
       if (act) store_u16<CPL>(o, other);
-    } else if (act) {
+    } else if (act && !(HALF && ((FAM == 3 ? at.x : at.y) & 1))) {
       VecW<CPL, S8>::put(o, L);
     }
     at.next(dp, dx, dy, xw, xs, W);
@@ -205,7 +207,7 @@ __global__ void __launch_bounds__(256) k_lines(const __grid_constant__ LineArgs 
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-template <int CPL, bool S8, int FAM, bool BANDED, bool ADD = false>
+template <int CPL, bool S8, int FAM, bool BANDED, bool ADD = false, bool HALF = false>
 static cudaError_t launch_family(const LineArgs &a, int nf, int dirs, bool overlap, cudaStream_t s) {
   constexpr int kWarp = kLineAhead * 32 * CPL * (ADD ? 3 : 1) + (BANDED ? kGW * kGL * CPL * 2 : 0);
   constexpr int kFit = 224 * 1024 / kWarp, kMaxWarps = kFit < 8 ? kFit : 8;   // (the ADD walks' rings are three times as long)
@@ -215,7 +217,7 @@ static cudaError_t launch_family(const LineArgs &a, int nf, int dirs, bool overl
   cfg.blockDim = dim3(32 * warps);
   cfg.dynamicSmemBytes = warps * kWarp;
   static bool done[64] = {};
-  const cudaError_t e = smem_optin(k_lines<CPL, S8, FAM, BANDED, ADD>, kMaxWarps * kWarp, done);
+  const cudaError_t e = smem_optin(k_lines<CPL, S8, FAM, BANDED, ADD, HALF>, kMaxWarps * kWarp, done);
   if (e != cudaSuccess) return e;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -223,7 +225,7 @@ static cudaError_t launch_family(const LineArgs &a, int nf, int dirs, bool overl
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = overlap ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k_lines<CPL, S8, FAM, BANDED, ADD>, a);
+  return cudaLaunchKernelEx(&cfg, k_lines<CPL, S8, FAM, BANDED, ADD, HALF>, a);
 }
 
 // Where a family's down and up vectors of a pixel lie.  S8: side by side,
@@ -252,8 +254,7 @@ static cudaError_t launch_walks(const KParams &k, const Buffers &b, int nf, cuda
   a.k = k;
   if (BANDED) a.k.D = k.Dp;                      // cells are band positions
   a.cost = b.cost;
-  a.sc.p1x2 = (uint32_t)k.p1 * 0x10001u;
-  a.sc.dpx2 = (uint32_t)(k.p2 - k.p1) * 0x10001u;
+  a.sc = step_consts(k);
   a.gate = b.gate;
   a.lo = b.band_lo;
   // the first launch waits for the cost volume as usual; the others may start
@@ -271,6 +272,9 @@ static cudaError_t launch_walks(const KParams &k, const Buffers &b, int nf, cuda
       e = launch_family<CPL, S8, F, BANDED>(a, nf, 1, false, s);
       a.dir = 1;
       if (e == cudaSuccess) e = launch_family<CPL, S8, F, BANDED, true>(a, nf, 1, false, s);
+    } else if constexpr (S8 && !BANDED && (CPL == 16 || CPL == 24)) {
+      e = k.half ? launch_family<CPL, S8, F, BANDED, false, true>(a, nf, 2, overlap, s)
+                 : launch_family<CPL, S8, F, BANDED>(a, nf, 2, overlap, s);
     } else {
       e = launch_family<CPL, S8, F, BANDED>(a, nf, 2, overlap, s);
     }

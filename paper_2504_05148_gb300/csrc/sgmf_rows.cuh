@@ -328,8 +328,7 @@ cudaError_t launch_rows_t(const KParams &k, const Buffers &b, int nf, cudaStream
   a.dprime = b.dprime;
   a.dsub = k.subpixel ? b.dsub : nullptr;
   a.dbg_sum = b.dbg_sum;
-  a.sc.p1x2 = (uint32_t)k.p1 * 0x10001u;
-  a.sc.dpx2 = (uint32_t)(k.p2 - k.p1) * 0x10001u;
+  a.sc = step_consts(k);
   a.gate = b.gate;
   for (int i = 0; i < 2; ++i) {
     a.vec[i] = reinterpret_cast<const uint8_t *>(b.part[i]);

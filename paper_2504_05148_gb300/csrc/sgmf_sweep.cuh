@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(32 * SweepCfg<CPL>::kMaxWarps, 1) k_sweep(cons
   // one Eq. 2 step from predecessor (pr, mp) on costs Cc: the new vector and its min
   auto move = [&](uint32_t(&o)[NW], uint32_t &mo, const uint32_t(&pr)[NW], uint32_t mp, const uint32_t(&Cc)[NW]) {
     copy_vec<NW>(o, pr);
-    step<NW>(o, Cc, mp, sc, none);
+    step<NW, false, (NW < 8)>(o, Cc, mp, sc, none);
     mo = group_min<NW>(o);
   };
   bool ok = true;
@@ -474,8 +474,7 @@ cudaError_t launch_sweep_t(const KParams &k, const Buffers &b, int nf, cudaStrea
   a.sum[1] = reinterpret_cast<uint8_t *>(b.part[1]);
   a.err = b.err;
   a.gate = b.gate;
-  a.sc.p1x2 = (uint32_t)k.p1 * 0x10001u;
-  a.sc.dpx2 = (uint32_t)(k.p2 - k.p1) * 0x10001u;
+  a.sc = step_consts(k);
   a.strip = kGW * warps * CF::P;
   cudaLaunchAttribute attr[1];
   cudaLaunchConfig_t cfg = sweep_config<CPL>(nf, ctas, warps, s, attr);

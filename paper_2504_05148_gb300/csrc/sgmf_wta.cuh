@@ -34,27 +34,43 @@ struct WtaArgs {
   Buffers b;                    // frame 0's maps (d*, d', d-sub, row ORs, gate)
   const uint8_t *vec[kMaxWtaVec];   // frame 0's vectors, 2 Dp bytes per pixel
   size_t vec_frame[kMaxWtaVec];     // bytes from one frame to the next
+  const uint8_t *cost;          // HALF: frame 0's cost volume
+  StepConsts sc;                // HALF
   uint16_t *dbg_sum;            // frame 0's S (u16 vectors), or null
   int16_t *out;
 };
 
-// NP: pairs of byte vectors side by side; NS: u16 vectors (after the pairs)
-template <int CPL, int NP, int NS>
+// NP: pairs of byte vectors side by side; NS: u16 vectors (after the pairs);
+// HALF: the cost bytes too (after the vectors)
+template <int CPL, int NP, int NS, bool HALF>
 struct WtaCfg {
-  static constexpr int Dp = kGL * CPL, k8 = 32 * CPL, NV = NP + NS, kSlot = 2 * NV * k8;
-  // slots: one step each, about 16 KB a warp (at least 2)
-  static constexpr int R = kSlot * 8 <= 16384 ? 8 : (kSlot * 4 <= 16384 ? 4 : 2);
+  static constexpr int Dp = kGL * CPL, k8 = 32 * CPL, NV = NP + NS, kSlot = (2 * NV + (HALF ? 1 : 0)) * k8;
+  // slots: one step each, about 16 KB a warp (at least 2; HALF, which computes
+  // more per step and needs the warps: about 12 KB)
+  static constexpr int R = HALF ? (kSlot * 4 <= 12288 ? 4 : (kSlot * 3 <= 16384 ? 3 : 2))
+                                : (kSlot * 8 <= 16384 ? 8 : (kSlot * 4 <= 16384 ? 4 : 2));
   // at most 8 warps a CTA, and what the shared memory of the widest row leaves
   static constexpr int kFit = (226 * 1024 - kMaxDim * 8) / (R * kSlot), kMaxWarps = kFit < 8 ? kFit : 8;
   static_assert(kMaxWarps >= 1, "a warp's ring fits beside the widest row");
-  static int warps(int W) { return max(1, min(kMaxWarps, (W + 319) / 320)); }   // segments of about 80 pixels
+  // segments of about 80 pixels; HALF: two CTAs a SM at least
+  static int warps(int W) {
+    int n = max(1, min(kMaxWarps, (W + 319) / 320));
+    if (HALF) n = max(1, min(n, (112 * 1024 - W * 8) / (R * kSlot)));
+    return n;
+  }
   // the rings, the row's d' keys (u32), d* and the list of undecided pixels (u16)
   static int smem(int W) { return warps(W) * R * kSlot + (W + 3) / 4 * 4 * 8; }
 };
 
-template <int CPL, int NP, int NS, bool BANDED>
+// HALF: the walks left the vectors of odd rows (rows family: of odd columns)
+// out.  A direction's vector there is one step of Eq. 2 from its predecessor,
+// which lies in an even row (column) and was stored.  At D = 128 the kernel then
+// executes 565 instructions per 512 cells instead of 173 and is ALU-bound (78 %
+// of the pipe): 8 frames of 1242 x 375 605 -> 760 us, the walks 1185 -> 857.
+template <int CPL, int NP, int NS, bool BANDED, bool HALF>
 __global__ void __launch_bounds__(256) k_wta(const __grid_constant__ WtaArgs a) {
-  using CF = WtaCfg<CPL, NP, NS>;
+  using CF = WtaCfg<CPL, NP, NS, HALF>;
+  static_assert(!HALF || (NS == 0 && !BANDED), "HALF: byte vectors of the full range");
   constexpr int NW = CPL / 2, Dp = CF::Dp, R = CF::R, NV = CF::NV;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ int n_list;
@@ -75,33 +91,60 @@ __global__ void __launch_bounds__(256) k_wta(const __grid_constant__ WtaArgs a) 
     // the group's segment [x0, x1): equal lengths, the last ones may be short or empty
     int seg = (W + kGW * nwarp - 1) / (kGW * nwarp);
     if constexpr (BANDED) seg = (seg + kBandTile - 1) / kBandTile * kBandTile;
+    if constexpr (HALF) seg = (seg + 1) / 2 * 2;     // segments start at even columns
     const int gi = warp * kGW + grp;
     const int x0 = min(gi * seg, W), x1 = min(x0 + seg, W);
     uint8_t *ring = smem + warp * R * CF::kSlot;
     const uint32_t ring_s = smem_u32(ring);
     const uint8_t *pv[NV];
+    [[maybe_unused]] const uint8_t *pc = nullptr;
+    [[maybe_unused]] const bool odd_row = HALF && (y & 1);
 #pragma unroll
     for (int j = 0; j < NV; ++j)
-      pv[j] = a.vec[j] + f * a.vec_frame[j] + (row + min(x0, W - 1)) * 2 * Dp +
+      pv[j] = a.vec[j] + f * a.vec_frame[j] + (row + (HALF ? 0 : min(x0, W - 1))) * 2 * Dp +
               lig * (j < NP ? Vec8<CPL>::kLane : Vec16<CPL>::kLane);
-    auto copy = [&](uint32_t slot, bool move) {
+    if constexpr (HALF) pc = a.cost + f * frame_cells(a.k) + row * Dp + lig * Vec8<CPL>::kLane;
+    // step t's copies into a slot.  A group past its segment's end copies the
+    // segment's last pixel again (HALF: goes on, to the row's last)
+    auto copy = [&](uint32_t slot, int t) {
+      if constexpr (HALF) {
+        const int x = min(x0 + t, W - 1);
+        copy8<CPL>(slot + 2 * NP * CF::k8, lane, pc + (size_t)x * Dp);
+        // the rows' vectors of an even column, or right -> left the next column's
+        if (!(t & 1)) copy8<CPL>(slot, lane, pv[0] + (size_t)x * (2 * Dp));
+        copy8<CPL>(slot + CF::k8, lane, pv[0] + (size_t)(t & 1 ? min(x + 1, W - 1) : x) * (2 * Dp) + Dp);
+        // where the predecessors lie: the row above (the down directions) and
+        // below (the up ones; clamped at the last row, the vector is then not used)
+        const int xm = max(x - 1, 0), xp = min(x + 1, W - 1);
+        const ptrdiff_t up_row = odd_row ? -(ptrdiff_t)W : 0, down_row = odd_row && y + 1 < a.k.H ? W : up_row;
 #pragma unroll
-      for (int j = 0; j < NV; ++j) {
-        const uint32_t d = slot + 2 * j * CF::k8;
-        if (j < NP) {
-          copy8<CPL>(d, lane, pv[j]);
-          copy8<CPL>(d + CF::k8, lane, pv[j] + Dp);
-        } else {
-          copy16<CPL>(d, lane, pv[j]);
+        for (int j = 1; j < NP; ++j) {
+          const int xd = !odd_row || j == 1 ? x : (j == 2 ? xm : xp), xu = !odd_row || j == 1 ? x : (j == 2 ? xp : xm);
+          copy8<CPL>(slot + 2 * j * CF::k8, lane, pv[j] + (up_row + xd) * (2 * Dp));
+          copy8<CPL>(slot + (2 * j + 1) * CF::k8, lane, pv[j] + (down_row + xu) * (2 * Dp) + Dp);
         }
-        if (move) pv[j] += 2 * Dp;
+      } else {
+#pragma unroll
+        for (int j = 0; j < NV; ++j) {
+          const uint32_t d = slot + 2 * j * CF::k8;
+          if (j < NP) {
+            copy8<CPL>(d, lane, pv[j]);
+            copy8<CPL>(d + CF::k8, lane, pv[j] + Dp);
+          } else {
+            copy16<CPL>(d, lane, pv[j]);
+          }
+          if (x0 + t + 1 < x1) pv[j] += 2 * Dp;
+        }
       }
     };
-    // a group past its segment's end copies the segment's last pixel again
     for (int t = 0; t < R; ++t) {
-      copy(ring_s + t * CF::kSlot, x0 + t + 1 < x1);
+      copy(ring_s + t * CF::kSlot, t);
       cp_commit();
     }
+    [[maybe_unused]] uint32_t z[CPL / 4] = {};
+    [[maybe_unused]] Raw8<CPL> right = {};       // HALF: the left -> right vector of the even column before
+    [[maybe_unused]] const Edges none = no_neighbours(lig);
+    if constexpr (HALF) pad_bytes<CPL>(D, lig, z);
     uint32_t kb[NW];                             // the keys' low bytes (d) and the padding's high ones
     [[maybe_unused]] const int16_t *lo_row = nullptr;
     [[maybe_unused]] int lo = 0;                 // the band start of the tile
@@ -150,27 +193,78 @@ __global__ void __launch_bounds__(256) k_wta(const __grid_constant__ WtaArgs a) 
           __syncwarp();
         }
       }
-      cp_wait<R - 1>();
       uint32_t Sm[NW];
-#pragma unroll
-      for (int w = 0; w < NW; ++w) Sm[w] = 0u;
-#pragma unroll
-      for (int j = 0; j < NV; ++j) {
-        const uint8_t *v = ring + base + 2 * j * CF::k8;
-        uint32_t T[NW];
-        if (j < NP) {
-          uint32_t U[NW];
-          slot8<CPL>(v, lane, z0, T);
-          slot8<CPL>(v + CF::k8, lane, z0, U);
-#pragma unroll
-          for (int i = 0; i < NW; ++i) Sm[i] = j == 0 ? T[i] + U[i] : Sm[i] + T[i] + U[i];
+      if constexpr (HALF) {
+        cp_wait<R - 1>();
+        const uint8_t *v = ring + base;
+        uint32_t C[NW], A[NW], B[NW];
+        slot8<CPL>(v + 2 * NP * CF::k8, lane, z, C);
+        // A and B: two predecessors' vectors -> their directions' vectors here
+        auto step2 = [&]() {
+          uint32_t ma, mb;
+          group_min2<NW>(A, B, ma, mb);
+          step<NW>(A, C, ma, a.sc, none);
+          step<NW>(B, C, mb, a.sc, none);
+        };
+        if (!(t & 1)) {
+          slot_raw8<CPL>(v, lane, right);
+          expand8<CPL>(right, z0, A);
+          slot8<CPL>(v + CF::k8, lane, z0, B);
         } else {
-          slot16<CPL>(v, lane, T);
+          Raw8<CPL> left;
+          slot_raw8<CPL>(v + CF::k8, lane, left);
+          if (x + 1 >= W) left = {};             // the path right -> left starts here
+          expand8<CPL>(right, z, A);
+          expand8<CPL>(left, z, B);
+          step2();
+        }
 #pragma unroll
-          for (int i = 0; i < NW; ++i) Sm[i] = j == 0 ? T[i] : Sm[i] + T[i];
+        for (int w = 0; w < NW; ++w) Sm[w] = A[w] + B[w];
+        if (!odd_row) {
+#pragma unroll
+          for (int j = 1; j < NP; ++j) {
+            slot8<CPL>(v + 2 * j * CF::k8, lane, z0, A);
+            slot8<CPL>(v + (2 * j + 1) * CF::k8, lane, z0, B);
+#pragma unroll
+            for (int w = 0; w < NW; ++w) Sm[w] += A[w] + B[w];
+          }
+        } else {
+          const bool last = y + 1 >= a.k.H;
+#pragma unroll
+          for (int j = 1; j < NP; ++j) {
+            Raw8<CPL> dn, up;
+            slot_raw8<CPL>(v + 2 * j * CF::k8, lane, dn);
+            slot_raw8<CPL>(v + (2 * j + 1) * CF::k8, lane, up);
+            // paths that start here: the predecessor lies outside the image
+            if (j == 2 ? x == 0 : (j == 3 && x == W - 1)) dn = {};
+            if (last || (j == 2 ? x == W - 1 : (j == 3 && x == 0))) up = {};
+            expand8<CPL>(dn, z, A);
+            expand8<CPL>(up, z, B);
+            step2();
+#pragma unroll
+            for (int w = 0; w < NW; ++w) Sm[w] += A[w] + B[w];
+          }
+        }
+      } else {
+        cp_wait<R - 1>();
+#pragma unroll
+        for (int j = 0; j < NV; ++j) {
+          const uint8_t *v = ring + base + 2 * j * CF::k8;
+          uint32_t T[NW];
+          if (j < NP) {
+            uint32_t U[NW];
+            slot8<CPL>(v, lane, z0, T);
+            slot8<CPL>(v + CF::k8, lane, z0, U);
+#pragma unroll
+            for (int i = 0; i < NW; ++i) Sm[i] = j == 0 ? T[i] + U[i] : Sm[i] + T[i] + U[i];
+          } else {
+            slot16<CPL>(v, lane, T);
+#pragma unroll
+            for (int i = 0; i < NW; ++i) Sm[i] = j == 0 ? T[i] : Sm[i] + T[i];
+          }
         }
       }
-      copy(ring_s + base, x + R + 1 < x1);
+      copy(ring_s + base, t + R);
       cp_commit();
       base = base + CF::kSlot == R * CF::kSlot ? 0 : base + CF::kSlot;
       if (dbg != nullptr && act) store_u16<CPL>(dbg + (size_t)x * Dp * 2, Sm);
@@ -254,14 +348,14 @@ __global__ void __launch_bounds__(256) k_wta(const __grid_constant__ WtaArgs a) 
   }
 }
 
-template <int CPL, int NP, int NS, bool BANDED>
+template <int CPL, int NP, int NS, bool BANDED, bool HALF = false>
 static cudaError_t launch_wta_v(const WtaArgs &a, int nf, cudaStream_t s) {
-  using CF = WtaCfg<CPL, NP, NS>;
+  using CF = WtaCfg<CPL, NP, NS, HALF>;
   static bool done[64] = {};
   const int most = CF::kMaxWarps * CF::R * CF::kSlot + kMaxDim * 8;
-  cudaError_t e = smem_optin(k_wta<CPL, NP, NS, BANDED>, most, done);
+  cudaError_t e = smem_optin(k_wta<CPL, NP, NS, BANDED, HALF>, most, done);
   if (e != cudaSuccess) return e;
-  k_wta<CPL, NP, NS, BANDED><<<dim3(a.k.H, nf), 32 * CF::warps(a.k.W), CF::smem(a.k.W), s>>>(a);
+  k_wta<CPL, NP, NS, BANDED, HALF><<<dim3(a.k.H, nf), 32 * CF::warps(a.k.W), CF::smem(a.k.W), s>>>(a);
   return cudaGetLastError();
 }
 
@@ -270,6 +364,8 @@ static cudaError_t launch_wta_b(const KParams &k, const Buffers &b, int nf, int1
   WtaArgs a = {};
   a.k = k;
   a.b = b;
+  a.cost = b.cost;
+  a.sc = step_consts(k);
   a.dbg_sum = b.dbg_sum;
   a.out = out;
   int n = 0;
@@ -287,6 +383,9 @@ static cudaError_t launch_wta_b(const KParams &k, const Buffers &b, int nf, int1
     add(v[0], frame[0]);
     if (!S8) add(v[1], frame[1]);
   }
+  if constexpr (S8 && !BANDED && (CPL == 16 || CPL == 24))
+    if (k.half)
+      return nfam == 3 ? launch_wta_v<CPL, 4, 0, BANDED, true>(a, nf, s) : launch_wta_v<CPL, 2, 0, BANDED, true>(a, nf, s);
   if constexpr (S8)
     return nfam == 3 ? launch_wta_v<CPL, 4, 0, BANDED>(a, nf, s) : launch_wta_v<CPL, 2, 0, BANDED>(a, nf, s);
   else

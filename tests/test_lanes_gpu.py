@@ -55,3 +55,40 @@ def test_line_and_winner_kernels(gpu, W, H, D, p2):
                                     dict(num_paths=4, p2=300, subpixel=1)])
 def test_winner_kernel_options(gpu, params):
     _check(scenes.random_small(771, 402, 23, 100), S.Params(**params), n=2)
+
+
+# calls of at least 100 M cells (200 M with four paths) at Dp = 128 and 192: the
+# walks store every second row's (column's) vectors.  Small frames in large
+# batches put the parities and borders where they can go wrong: one row, two
+# columns, odd and even sizes, segments that end on odd columns
+@pytest.mark.parametrize("W,H,D,params", [
+    (2, 100, 128, {}), (200, 1, 128, {}), (199, 2, 65, {}), (41, 40, 192, {}), (321, 7, 129, {}), (17, 33, 100, {}),
+    (640, 9, 128, dict(subpixel=1)), (162, 15, 192, dict(num_paths=4)), (83, 24, 128, dict(num_paths=4)),
+    (96, 31, 128, dict(consistency=S.SGMF_CHECK_LIDAR))])
+def test_half_stored_vectors(gpu, W, H, D, params):
+    import torch
+    dev = torch.device("cuda:0")
+    p = S.Params(**params)
+    dp = 128 if D <= 128 else 192
+    n = -(-(200_000_000 if p.num_paths == 4 else 100_000_000) // (W * H * dp))
+    assert 3 <= n <= 4096
+    scs = [scenes.random_small(8800 + i, W, H, D) for i in range(3)]
+    rep = lambda name: torch.from_numpy(np.stack([getattr(s, name) for s in scs])).to(dev)[
+        torch.arange(n, device=dev) % 3].contiguous()
+    ctx = S.Context(W, H, D, p, max_batch=n)
+    try:
+        ctx.set_debug(True)
+        out = torch.empty((n, H, W), dtype=torch.int16, device=dev)
+        ctx.compute(rep("left"), rep("right"), rep("lidar"), out)
+        ctx.sync()
+        total = ctx.stage(S.SGMF_STAGE_SUM)
+        dprime = ctx.stage(S.SGMF_STAGE_DPRIME)
+        got = out.cpu().numpy()
+    finally:
+        ctx.close()
+    for i, s in enumerate(scs):
+        o = oracle.compute(s.left, s.right, s.lidar, D, oracle.Params(**vars(p)), volumes=i == 0)
+        if i == 0:
+            np.testing.assert_array_equal(total.astype(np.int64), o.sum.astype(np.int64))
+            np.testing.assert_array_equal(dprime, o.dprime)
+        assert (got[i::3] == o.out).all(), f"frame {i}"
