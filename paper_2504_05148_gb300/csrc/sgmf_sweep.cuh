@@ -27,9 +27,11 @@
 // cluster scope inside the row loop.
 //
 // Cost rows arrive by bulk copies (one per row and CTA: the strip's pixels
-// are contiguous) into a ring of R stages, two rows ahead.  Every mbarrier
+// are contiguous) into a ring of R stages, R - 2 rows ahead.  Every mbarrier
 // wait is bounded (the error word records a timeout); the two cluster
 // barriers, at the start and the end, are executed by every thread.
+//
+// What bounds it is the ALU pipe (u16x2 minima and adds at half rate).
 #pragma once
 
 #include "sgmf_lines.cuh"
@@ -52,13 +54,16 @@ struct SweepArgs {
 template <int CPL>
 struct SweepCfg {
   static constexpr int Dp = kGL * CPL, NW = CPL / 2;
-  // pixels per group: 3 P NW words of path costs a lane, at most 96
+  // pixels per group: 3 P NW words of path costs a lane, at most 96.  (Two CTAs
+  // a SM of 6 warps and 168 registers, ring of 3 rows: 32 frames of 1242 x 375,
+  // D = 128 3.30 against 3.00 ms; more warps do not help, the ALU pipe is full)
   static constexpr int P = CPL <= 16 ? 4 : 2;
   static constexpr int kMaxWarps = CPL <= 16 ? 8 : 10;
   static constexpr int kMaxCluster = 16;         // CTAs per cluster (above 8: non-portable)
   static constexpr int kMaxRow = CPL <= 16 ? 2048 : 1280;   // pixels of a row the sweep takes
   static constexpr int R = 4;                    // ring stages (rows)
-  static constexpr int kBars = R + 6;            // mbarriers (and padding: the slots start on 16 bytes)
+  static constexpr int kBars = (R + 6) / 2 * 2;  // R + 5 mbarriers, padded: the slots start on 16 bytes
+  static_assert(kBars >= R + 5 && kBars % 2 == 0, "room for the barriers, and aligned slots");
   static constexpr int kSlot = (NW + 1) * kGL;   // words of one exchanged vector: NW words + m, per lane
   // at least kExclusive bytes: one CTA per SM, so that the clusters the
   // device holds at once are the SMs the sweep occupies
@@ -226,11 +231,12 @@ __global__ void __launch_bounds__(32 * SweepCfg<CPL>::kMaxWarps, 1) k_sweep(cons
   const uint32_t keep_in_l = xg == 0 ? 0u : 0xffffffffu;
   // warps whose groups touch neither border need none of the masks below
   const bool plain = __all_sync(kAll, xg > 0 && xg + P < W);
-  // one Eq. 2 step from predecessor (pr, mp) on costs Cc: the new vector and its min
-  auto move = [&](uint32_t(&o)[NW], uint32_t &mo, const uint32_t(&pr)[NW], uint32_t mp, const uint32_t(&Cc)[NW]) {
+  // one Eq. 2 step from predecessor (pr, mp) on costs Cc: the new vector.  Its
+  // min follows, two vectors at a time (one pass of shuffles for both: 32 frames
+  // of 1242 x 375, D = 128 3.08 -> 3.00 ms)
+  auto move = [&](uint32_t(&o)[NW], const uint32_t(&pr)[NW], uint32_t mp, const uint32_t(&Cc)[NW]) {
     copy_vec<NW>(o, pr);
     step<NW, false, (NW < 8)>(o, Cc, mp, sc, none);
-    mo = group_min<NW>(o);
   };
   bool ok = true;
   auto bounded = [&](uint64_t *bar, uint32_t parity) {
@@ -265,8 +271,9 @@ __global__ void __launch_bounds__(32 * SweepCfg<CPL>::kMaxWarps, 1) k_sweep(cons
         for (int w = 0; w < NW; ++w) pr[w] &= kr;
         mpr &= kr;
       }
-      move(eL, meL, DL[P - 2], mL[P - 2], CP);
-      move(eR, meR, pr, mpr, C0);
+      move(eL, DL[P - 2], mL[P - 2], CP);
+      move(eR, pr, mpr, C0);
+      group_min2<NW>(eL, eR, meL, meR);
     }
     // the vectors entering this group from the previous row
     uint32_t inL[NW], inR[NW], minL = 0u, minR = 0u;
@@ -285,7 +292,8 @@ __global__ void __launch_bounds__(32 * SweepCfg<CPL>::kMaxWarps, 1) k_sweep(cons
       get(1, par, inR, minR);
     }
     // the ring stage of row t - 2 is free: every warp finished that row before its row t - 1 arrival
-    if (threadIdx.x == 0 && issued < H && issued <= t + 2) issue(issued);
+    // (row t - 1 may still be read), so rows up to t - 2 + R may be on their way
+    if (threadIdx.x == 0 && issued < H && issued <= t - 2 + R) issue(issued);
     if (t + 1 < H) {
       // row t's outgoing vectors (the last row's have no reader)
       const int par = t & 1;
@@ -307,7 +315,7 @@ __global__ void __launch_bounds__(32 * SweepCfg<CPL>::kMaxWarps, 1) k_sweep(cons
     }
     uint32_t carry[NW], mcarry = mL[0];
     copy_vec<NW>(carry, DL[0]);
-    move(DL[0], mL[0], inL, minL, C0);
+    move(DL[0], inL, minL, C0);
 #pragma unroll
     for (int i = 0; i < P; ++i) {
       uint32_t C[NW];
@@ -317,14 +325,13 @@ __global__ void __launch_bounds__(32 * SweepCfg<CPL>::kMaxWarps, 1) k_sweep(cons
         copy_vec<NW>(C, CP);
       else
         load_u8<CPL>(st + i * Dp, z, C);
-      uint32_t mtmp;
-      move(V[i], mtmp, V[i], mV[i], C);
-      mV[i] = mtmp;
+      move(V[i], V[i], mV[i], C);
       if (i >= 1 && i <= P - 2) {
         uint32_t nxt[NW];
         const uint32_t mnxt = mL[i];
         copy_vec<NW>(nxt, DL[i]);
-        move(DL[i], mL[i], carry, mcarry, C);
+        move(DL[i], carry, mcarry, C);
+        group_min2<NW>(V[i], DL[i], mV[i], mL[i]);
         copy_vec<NW>(carry, nxt);
         mcarry = mnxt;
         uint32_t pr[NW], mpr = mR[i + 1];
@@ -335,14 +342,17 @@ __global__ void __launch_bounds__(32 * SweepCfg<CPL>::kMaxWarps, 1) k_sweep(cons
           for (int w = 0; w < NW; ++w) pr[w] &= ki;
           mpr &= ki;
         }
-        move(DR[i], mR[i], pr, mpr, C);
+        move(DR[i], pr, mpr, C);
+        if (i % 2 == 0) group_min2<NW>(DR[i - 1], DR[i], mR[i - 1], mR[i]);   // (i = 1 waits for i = 2)
       } else if (i == 0) {
+        group_min2<NW>(V[0], DL[0], mV[0], mL[0]);
         copy_vec<NW>(DR[0], eR);
         mR[0] = meR;
       } else {
         copy_vec<NW>(DL[P - 1], eL);
         mL[P - 1] = meL;
-        move(DR[P - 1], mR[P - 1], inR, minR, C);
+        move(DR[P - 1], inR, minR, C);
+        group_min2<NW>(V[P - 1], DR[P - 1], mV[P - 1], mR[P - 1]);
       }
       uint32_t sum[NW];
 #pragma unroll
