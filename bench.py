@@ -55,21 +55,22 @@ TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic_kitti_1242x375_d128.txt")
 
 # Algorithmic work of each kernel for V = W*H*D cells and N = W*H pixels.
 # bytes: data the stage must read and write in HBM given its inputs and outputs
-#        (spills and re-reads chosen by the implementation are not counted);
+#        (re-reads chosen by the implementation are not counted);
 # ops:   scalar integer operations of the method (Eq. 2: 2 adds of P1, 3 mins,
 #        1 add of C, 1 subtraction of m and 1 min toward the next m = 8 per cell
 #        and direction; the path sum 1 add per cell and direction; WTA 2 mins per cell).
 def algorithmic(name: str, V: int, N: int, num_paths: int = 8, sweep: bool = False):
     if name == "agg_lines":
         # the cost volume read once, one byte vector per direction written
-        dirs = num_paths - 2
-        return {"bytes": V * 1 + (dirs // 2) * 2 * V, "ops": 8 * dirs * V + (dirs // 2) * V}
+        return {"bytes": V * 1 + num_paths * V, "ops": 8 * num_paths * V}
     if name == "agg_sweep":
         # the cost volume read once, two u16 sums of three directions written
         return {"bytes": V * 1 + 2 * 2 * V, "ops": 8 * 6 * V + 4 * V}
     if name == "agg_rows_wta":
-        fams = 2 if sweep else (num_paths - 2) // 2     # u16 sums (sweep) or byte-vector pairs
-        return {"bytes": V * 1 + fams * 2 * V + 4 * N, "ops": 8 * 2 * V + (2 + fams) * V + 2 * V}
+        if not sweep:                    # every direction's byte vectors read, summed, WTA
+            return {"bytes": num_paths * V + 4 * N, "ops": num_paths * V + 2 * V}
+        # the row walks, and two u16 sums of three directions read
+        return {"bytes": V * 1 + 2 * 2 * V + 4 * N, "ops": 8 * 2 * V + 4 * V + 2 * V}
     if name == "cost":
         return {"bytes": V + 4 * N * 2 + 2 * N, "ops": 4 * V}
     return None

@@ -408,7 +408,7 @@ typedef struct {
                              segments of up to 1024 pixels) */
     int32_t sweep;        /* 1: the six vertical and diagonal directions run as two
                              row-synchronous sweeps of a thread-block cluster per
-                             frame (one launch) instead of the three line kernels
+                             frame (one launch) instead of their line walks
                              (line_warps is then unused).  0 (default) or 1; 1 needs
                              a row of at most 16 CTAs x 128 pixels (Dp <= 128) or
                              16 x 80 pixels (Dp > 128; banded: 16 x 160) and

@@ -2,7 +2,7 @@
 // restricted to a disparity band [lo_p, lo_p + B) per pixel, lo_p constant on
 // kBandTile x kBandTile pixel tiles.  Ingest, census, semidensification and
 // the check are the plain kernels; the cost (here) and the aggregation with
-// its WTA (sgmf_aggregate.cuh, BANDED variants) work on the bands.
+// its WTA (sgmf_lines.cuh, sgmf_wta.cuh, BANDED variants) work on the bands.
 #include <cstdint>
 
 #include "sgmf_cost.cuh"

@@ -654,8 +654,9 @@ cudaError_t launch_semidense(const KParams &k, const Buffers &b, int nf, cudaStr
 // each lane the same DPL disparities of all four: the P + DPL - 1 window
 // entries cR(x - d) they need are consecutive and start on a vector boundary
 // (x - d0 is a multiple of 4 there), so a lane loads them with a few aligned
-// vector loads and indexes them with constants; a lane stores DPL cost bytes
-// a pixel, a warp's stores one contiguous row of the cost volume.  (Eight
+// vector loads and indexes them with constants; pairs of lanes exchange bytes for
+// the volume's lane order and each stores two of the four pixels, a warp's
+// stores contiguous rows of the cost volume.  (Eight
 // pixels a step, for fewer loop and load instructions, ran 14 % slower: the
 // registers they need halve the resident warps.)
 template <typename CT, int DPL, bool SEMI>

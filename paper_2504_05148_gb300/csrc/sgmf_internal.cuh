@@ -8,8 +8,10 @@
 //                                           sparse disparity of the window is d
 //   cost C-bar      uint8  [F][H][W][Dp]   Dp = 32 * DPL >= D, cells d >= D hold 0;
 //                                           cells in group-lane order (sgmf_lanes.cuh)
-//   partial sums    u16    [F][H][W][Dp]   one per line family (vertical, two diagonals)
-//   spills          uint8/u16 [F][4][line][pos][Dp]  first-direction path costs of a line
+//   path costs      2 Dp bytes a pixel and line family (vertical, two diagonals): both
+//                                           directions' byte vectors, u16 vectors of one,
+//                                           or (the first two) the sweep's u16 sums
+//   spill           4 such regions: the rows' path costs, u16 vectors of the other directions
 // F is the number of frames a context holds (its batch capacity); every
 // kernel takes the frame from its last grid dimension.
 #pragma once
@@ -61,8 +63,8 @@ struct Buffers {   // base pointers of frame 0
   uint32_t *boxC;             // [MW][H][W] their row ORs only (|x' - x| <= r_c), radius r_c
   uint32_t *boxTmp;           // [F][MW][H][W] r_s row-pass results (scratch of the column pass)
   uint8_t *cost;              // [H][W][Dp]
-  uint16_t *part[3];          // [H][W][Dp]
-  void *spill;                // 4 regions (vertical, diag, anti-diag, rows) of H*W*Dp elements
+  uint16_t *part[3];          // path costs of a family (vertical, diagonals), or the sweep's sums
+  void *spill;                // 4 regions of 2 H*W*Dp bytes: path costs (family_vectors in sgmf_lines.cuh)
   uint16_t *dbg_sum;          // [H][W][Dp] or null
   int *err;                   // device error word
   int16_t *band_lo;           // banded mode: band start per tile, [frame][th][tw] (clamped copy)
