@@ -537,10 +537,27 @@ static sgmf_status front_stages(sgmf_ctx *c, int f0, int nf, const uint8_t *left
   return SGMF_OK;
 }
 
+// Whether the rows behind the sweep of nf frames are line walks, whose byte
+// vectors the winner kernel adds to the sweep's two sums, instead of the row
+// kernel and the check: as many launches, one more byte per cell and direction
+// written and read, but a chain of shorter steps.  It pays where few rows leave
+// that chain as the time: 8 frames of 1332 x 53, D = 124 (2.8 rows a SM) 1126 ->
+// 647 us, of 640 x 120, D = 128 (6.3) 485 -> 486, of 1242 x 200, D = 128 (10.5)
+// 1529 -> 1213.  Above 12 rows a SM either is
+// the faster one, the row kernel for 13 frames of 1242 x 375 (2907 against 2978 us)
+// and 12 of 320 x 240, D = 64 (474 against 490), and it stays.
+constexpr int kRowLinesPerSm = 12;
+static bool rows_as_lines(const sgmf_ctx *c, int nf) {
+  int sms = 0;
+  if (!c->spill8 || sm_count(&sms) != cudaSuccess) return false;
+  return (long)c->k.H * nf <= (long)kRowLinesPerSm * sms;
+}
+
 // What follows the cost volume (and, with the sweep, the sweep) for the nf
 // frames of b on stream s, down to the output.
-static sgmf_status finish(sgmf_ctx *c, const KParams &ka, const Buffers &b, int nf, int16_t *out, cudaStream_t s) {
-  if (ka.sweep) {
+static sgmf_status finish(sgmf_ctx *c, KParams ka, const Buffers &b, int nf, int16_t *out, cudaStream_t s) {
+  ka.rows_lines = ka.sweep && rows_as_lines(c, nf);
+  if (ka.sweep && !ka.rows_lines) {
     TIMED(c, "agg_rows_wta", s, launch_agg_rows(ka, b, nf, c->spill8, s));
     TIMED(c, "consistency", s, launch_consistency(c->k, b, nf, out, s));
     return SGMF_OK;
@@ -575,7 +592,7 @@ static int half_vectors(const sgmf_ctx *c, int n) {
 // KITTI frames, and 3 % slower at 64; the sweep slows by what they save.)
 static sgmf_status aggregate(sgmf_ctx *c, int n, int16_t *out, cudaStream_t s) {
   KParams ka = agg_params(c);
-  ka.half = half_vectors(c, n);
+  ka.half = ka.sweep ? 0 : half_vectors(c, n);
   const int m = ka.sweep ? sweep_part(c, n) : 0;
   if (m == 0) {
     if (ka.sweep) TIMED(c, "agg_sweep", s, launch_agg_sweep(ka, c->b, n, s));

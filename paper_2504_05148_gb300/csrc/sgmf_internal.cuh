@@ -50,6 +50,7 @@ struct KParams {
   int band;                   // banded mode: band width B (= Dp); 0 = the plain method
   int tw, th;                 // banded mode: band tiles per row / column
   uint32_t wait_census;       // poll limit of the census kernel's TMA wait (kWaitLimit by default)
+  int rows_lines;             // behind the sweep: the rows as line walks and the winner kernel (set per call)
   int half;                   // the line walks store half of the vectors (set per call)
   int gate_run;               // with Buffers::gate: a frame runs when its gate word equals this
 };

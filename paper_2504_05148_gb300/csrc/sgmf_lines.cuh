@@ -281,6 +281,7 @@ static cudaError_t launch_walks(const KParams &k, const Buffers &b, int nf, cuda
     overlap = true;
   };
   family(std::integral_constant<int, 3>{});
+  if (k.rows_lines) return e;                       // the other directions are the sweep's
   family(std::integral_constant<int, 0>{});
   if (k.num_paths == 8) {
     family(std::integral_constant<int, 1>{});

@@ -378,6 +378,11 @@ static cudaError_t launch_wta_b(const KParams &k, const Buffers &b, int nf, int1
   size_t frame[2];
   family_vectors(k, b, S8, 3, v, frame);
   add(v[0], frame[0]);                           // the rows: a pair of byte vectors, or their u16 sum
+  if constexpr (S8 && !BANDED)
+    if (k.rows_lines) {                          // the other directions: the sweep's two u16 sums
+      for (int i = 0; i < 2; ++i) add(reinterpret_cast<const uint8_t *>(b.part[i]), 2 * frame_cells(k));
+      return launch_wta_v<CPL, 1, 2, BANDED>(a, nf, s);
+    }
   for (int i = 0; i < nfam; ++i) {
     family_vectors(k, b, S8, i, v, frame);
     add(v[0], frame[0]);
