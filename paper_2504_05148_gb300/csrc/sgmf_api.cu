@@ -543,9 +543,9 @@ static sgmf_status front_stages(sgmf_ctx *c, int f0, int nf, const uint8_t *left
 // written and read, but a chain of shorter steps.  It pays where few rows leave
 // that chain as the time: 8 frames of 1332 x 53, D = 124 (2.8 rows a SM) 1126 ->
 // 647 us, of 640 x 120, D = 128 (6.3) 485 -> 486, of 1242 x 200, D = 128 (10.5)
-// 1529 -> 1213.  Above 12 rows a SM either is
-// the faster one, the row kernel for 13 frames of 1242 x 375 (2907 against 2978 us)
-// and 12 of 320 x 240, D = 64 (474 against 490), and it stays.
+// 1529 -> 1213.  Above 12 rows a SM it depends on the shape, and the row kernel
+// stays: 13 frames of 1242 x 375 2907 against 2978 us, 12 of 320 x 240, D = 64 474
+// against 490, though 12 of 640 x 480, D = 64 1360 against 1277.
 constexpr int kRowLinesPerSm = 12;
 static bool rows_as_lines(const sgmf_ctx *c, int nf) {
   int sms = 0;
