@@ -422,9 +422,14 @@ __global__ void __launch_bounds__(128) k_bn_conv(const __grid_constant__ BnConvA
 // the pixels along K both are MN-major operands as they lie: for a fixed kx
 // the rows (ky, ci) of A are the twelve planes in turn (M = 128 with four
 // planes past them, whose rows are not read back), N = 32 channels of dY, and
-// the tile is eight MMAs of K = 16 pixels into the accumulator of kx.
+// a tile is at most eight MMAs of K = 16 pixels into the accumulator of kx.
+// Past a row's end dY = 0, and X = 0 for kx = 1, 2; for kx = 0 the first pixel
+// past it would meet the row's last X, and 0 times an infinity or NaN is no
+// zero: the kx = 0 operand of the 16 pixels in which the row ends is a copy of
+// its own, with X = 0 past the row.
 // (Transposing both through 2-byte shared-memory stores, 320 a pixel, took
-// 139 us where this takes 47 us: 16 x 94 x 311 pixels; the MMAs' operand reads
+// 139 us where this takes 44 us: 16 x 94 x 311 pixels, 47 before the steps past a
+// row's end were left out; the MMAs' operand reads
 // bound it, about 120 cycles each whatever the number of stages, loading warps
 // and CTAs.)  The accumulators and the bias gradient are written as
 // this CTA's partial sums; a second kernel adds the partials of all CTAs in a
@@ -435,7 +440,8 @@ constexpr int kWgThreads = 32 * kWgLoad;            // loading threads
 constexpr int kWgPlane = kCvM * 16;                 // a chunk plane of dY
 constexpr int kWgStage = 16 * kCvPlane;             // 12 planes of X, then the 4 of dY (and what M = 128 reads past them)
 static_assert(kCvX + 4 * kWgPlane <= kWgStage, "the planes fit the stage");
-constexpr int kWgSmem = kWgStages * kWgStage + 2 * kWgStages * 8 + 16;
+constexpr int kWgEnd = 16 * 256;                    // kx = 0 copy of a row's last step: 12 planes of 16 pixels (and as above)
+constexpr int kWgSmem = kWgStages * (kWgStage + kWgEnd) + 2 * kWgStages * 8 + 16;
 constexpr int kWgMaxCtas = 304;         // about two CTAs per SM
 constexpr int kWgPart = kBnK * 32 + 32; // one CTA's partial: dw [co][tap][ci], then db [co]
 // partial sums of one sgmf_bn_wgrad call (calls must not overlap on the GPU)
@@ -450,7 +456,8 @@ struct BnWgradArgs {
 
 __global__ void __launch_bounds__(kWgThreads + 32) k_bn_wgrad(const __grid_constant__ BnWgradArgs a) {
   extern __shared__ __align__(1024) uint8_t sm[];
-  uint64_t *full = reinterpret_cast<uint64_t *>(sm + kWgStages * kWgStage);   // a stage is filled
+  uint8_t *ends = sm + kWgStages * kWgStage;                                  // [stage] kx = 0 copies
+  uint64_t *full = reinterpret_cast<uint64_t *>(ends + kWgStages * kWgEnd);   // a stage is filled
   uint64_t *empty = full + kWgStages;                                         // its MMAs are done
   uint32_t *slot = reinterpret_cast<uint32_t *>(empty + kWgStages);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -497,12 +504,19 @@ __global__ void __launch_bounds__(kWgThreads + 32) k_bn_wgrad(const __grid_const
       if (t < nt) {
         if (t >= kWgStages && !wait(&empty[t % kWgStages], t / kWgStages - 1)) break;
         const uint32_t dst = smem_u32(sm) + t % kWgStages * kWgStage;
+        const int nv = min(kCvM, a.w - ld.x0), npx = (nv + 15) / 16 * 16;   // the tile's pixels; those of its steps
         bn_stage_rows<kWgThreads>(dst, a.x, ld, a.w, a.h);
+        if (nv != npx && tid < 12 * 16) {
+          const int p = tid >> 4, i = tid & 15, px = ld.x0 + npx - 17 + i, yy = ld.y + (p >> 2) - 1;   // plane, pixel
+          const bool in = (unsigned)yy < (unsigned)a.h && px >= 0 && px < a.w - 1;
+          const uint16_t *src = a.x + (((long long)ld.img * a.h + yy) * a.w + px) * kBnC + 8 * (p & 3);
+          cp_async16(smem_u32(ends) + t % kWgStages * kWgEnd + p * 256 + i * 16, in ? src : a.x, in);
+        }
         const uint16_t *src = a.dy + (((long long)ld.img * a.h + ld.y) * a.w + ld.x0) * kBnC + 8 * (tid & 3);
 #pragma unroll
         for (int s = 0; s < kY; ++s) {
           const int px = (tid >> 2) + s * (kWgThreads / 4);
-          const bool in = ld.x0 + px < a.w;
+          const bool in = px < nv;
           cp_async16(dst + kCvX + (tid & 3) * kWgPlane + px * 16, in ? src + px * kBnC : a.dy, in);
         }
         ld.next(a.w, a.h);
@@ -531,18 +545,24 @@ __global__ void __launch_bounds__(kWgThreads + 32) k_bn_wgrad(const __grid_const
     constexpr uint32_t idesc = idesc_bf16(128, 32, true);
     const uint32_t leader = elect_one();
     int issued = 0;
+    BnTile cur(tile0, tpr, a.h);
     for (int t = 0; t < nt; ++t) {
       if (!wait(&full[t % kWgStages], t / kWgStages)) break;
       tc_fence_after();
       const uint32_t x_0 = smem_u32(sm) + (t % kWgStages) * kWgStage;
       const uint64_t xd = sdesc(x_0, 128, kCvPlane), yd = sdesc(x_0 + kCvX, 128, kWgPlane);
+      const uint64_t ed = sdesc(smem_u32(ends) + (t % kWgStages) * kWgEnd, 128, 256);
+      const int nv = min(kCvM, a.w - cur.x0);
+      cur.next(a.w, a.h);
       // the three accumulators in turn: MMAs into one accumulator follow each other slower
 #pragma unroll
-      for (int s = 0; s < kCvM / 16; ++s)
+      for (int s = 0; s < kCvM / 16; ++s) {
+        if (16 * s >= nv) break;                     // (no pixel of the row)
 #pragma unroll
         for (int kx = 0; kx < 3; ++kx)
-          umma_bf16(tmem + 32 * kx, sdesc_at(xd, kx * 16 + s * 256), sdesc_at(yd, s * 256), idesc,
-                    (t > 0 || s > 0) ? 1u : 0u, leader);
+          umma_bf16(tmem + 32 * kx, kx == 0 && nv < 16 * s + 16 ? ed : sdesc_at(xd, kx * 16 + s * 256),
+                    sdesc_at(yd, s * 256), idesc, (t > 0 || s > 0) ? 1u : 0u, leader);
+      }
       umma_commit(&empty[t % kWgStages], leader);
       issued = t + 1;
     }
