@@ -207,14 +207,14 @@ constexpr int kCvSmem = kCvX + kBnB + 32 * 4 + 16;
 // Position of a tile: its first pixel x0 of row y of image img.
 struct BnTile {
   int x0, y, img;
-  __device__ __forceinline__ BnTile(long long tile, int tpr, int h) {
+  __device__ __forceinline__ BnTile(long long tile, int tpr, int h, int px = kCvM) {
     const long long row = tile / tpr;
-    x0 = (int)(tile - row * tpr) * kCvM;
+    x0 = (int)(tile - row * tpr) * px;
     img = (int)(row / h);
     y = (int)(row - (long long)img * h);
   }
-  __device__ __forceinline__ void next(int w, int h) {
-    x0 += kCvM;
+  __device__ __forceinline__ void next(int w, int h, int px = kCvM) {
+    x0 += px;
     if (x0 >= w) {
       x0 = 0;
       if (++y == h) {
@@ -224,31 +224,6 @@ struct BnTile {
     }
   }
 };
-
-// stage rows y - 1, y, y + 1, pixels x0 - 1 .. x0 + 128 of x as chunk planes
-// (zero outside the image), by THREADS threads: a thread keeps its chunk and
-// its pixels of each row, so that a piece is a compare and a copy
-template <int THREADS>
-__device__ __forceinline__ void bn_stage_rows(uint32_t dst, const uint16_t *x, const BnTile &t, int w, int h) {
-  const int j = threadIdx.x & 3, p0 = threadIdx.x >> 2;
-  const uint16_t *row = x + (((long long)t.img * h + t.y - 1) * w + t.x0 - 1) * kBnC;   // staged pixel 0 of row y - 1
-#pragma unroll
-  for (int ky = 0; ky < 3; ++ky) {
-    const bool row_in = (unsigned)(t.y + ky - 1) < (unsigned)h;
-    const uint16_t *src = row + ((long long)ky * w + p0) * kBnC + 8 * j;
-    const uint32_t d = dst + (ky * 4 + j) * kCvPlane + p0 * 16;
-#pragma unroll
-    for (int s = 0; s < kCvM * 4 / THREADS; ++s) {
-      const bool in = row_in && (unsigned)(t.x0 - 1 + p0 + s * (THREADS / 4)) < (unsigned)w;
-      cp_async16(d + s * (THREADS / 4) * 16, in ? src + s * (THREADS / 4) * kBnC : x, in);
-    }
-  }
-  if (threadIdx.x < 24) {                        // the last two pixels of each row
-    const int ky = threadIdx.x >> 3, px = kCvM + ((threadIdx.x >> 2) & 1);
-    const bool in = (unsigned)(t.y + ky - 1) < (unsigned)h && (unsigned)(t.x0 - 1 + px) < (unsigned)w;
-    cp_async16(dst + (ky * 4 + j) * kCvPlane + px * 16, in ? row + ((long long)ky * w + px) * kBnC + 8 * j : x, in);
-  }
-}
 
 __global__ void __launch_bounds__(128) k_bn_conv(const __grid_constant__ BnConvArgs a, int tiles) {
   extern __shared__ __align__(1024) uint8_t sm[];
@@ -417,31 +392,38 @@ __global__ void __launch_bounds__(128) k_bn_conv(const __grid_constant__ BnConvA
 
 // ---- weight gradient ---------------------------------------------------------------------
 // D[(tap, ci)][co] = sum over pixels of X[p + o_tap][ci] dY[p][co].  A CTA
-// reduces `chunks` tiles of 128 pixels of an image row.  X is staged as in the
+// reduces `chunks` stages of tiles of PX pixels of an image row.  X is staged as in the
 // forward pass (three rows, chunk planes) and dY as four chunk planes; with
 // the pixels along K both are MN-major operands as they lie: for a fixed kx
 // the rows (ky, ci) of A are the twelve planes in turn (M = 128 with four
 // planes past them, whose rows are not read back), N = 32 channels of dY, and
-// a tile is at most eight MMAs of K = 16 pixels into the accumulator of kx.
+// a tile is at most PX / 16 MMAs of K = 16 pixels into the accumulator of kx.
 // Past a row's end dY = 0, and X = 0 for kx = 1, 2; for kx = 0 the first pixel
 // past it would meet the row's last X, and 0 times an infinity or NaN is no
 // zero: the kx = 0 operand of the 16 pixels in which the row ends is a copy of
 // its own, with X = 0 past the row.
 // (Transposing both through 2-byte shared-memory stores, 320 a pixel, took
-// 139 us where this takes 44 us: 16 x 94 x 311 pixels, 47 before the steps past a
-// row's end were left out; the MMAs' operand reads
+// 154 us a call where this takes 56: 16 x 94 x 311 pixels, cold L2; the MMAs' operand reads
 // bound it, about 120 cycles each whatever the number of stages, loading warps
 // and CTAs.)  The accumulators and the bias gradient are written as
 // this CTA's partial sums; a second kernel adds the partials of all CTAs in a
 // fixed order, so that the gradient (and with it training) does not depend on
 // the order the CTAs finish in.
-constexpr int kWgStages = 3, kWgLoad = 8;           // loading warps; one more issues the MMAs
-constexpr int kWgThreads = 32 * kWgLoad;            // loading threads
-constexpr int kWgPlane = kCvM * 16;                 // a chunk plane of dY
-constexpr int kWgStage = 16 * kCvPlane;             // 12 planes of X, then the 4 of dY (and what M = 128 reads past them)
-static_assert(kCvX + 4 * kWgPlane <= kWgStage, "the planes fit the stage");
-constexpr int kWgEnd = 16 * 256;                    // kx = 0 copy of a row's last step: 12 planes of 16 pixels (and as above)
-constexpr int kWgSmem = kWgStages * (kWgStage + kWgEnd) + 2 * kWgStages * 8 + 16;
+template <int PIXELS, int TILES>
+struct WgCfg {
+  static constexpr int PX = PIXELS, kTiles = TILES;   // pixels of a tile, tiles of a stage
+  static constexpr int kStages = 3, kLoad = 8;        // loading warps; one more issues the MMAs
+  static constexpr int kThreads = 32 * kLoad, kGroup = kThreads / kTiles;   // loading threads, those of one tile
+  static constexpr int kXPlane = (PX + 2) * 16, kX = 12 * kXPlane, kYPlane = PX * 16;   // chunk planes of X and dY
+  static constexpr int kTile = 16 * kXPlane;          // 12 planes of X, then the 4 of dY (and what M = 128 reads past them)
+  static_assert(kX + 4 * kYPlane <= kTile && PX * 4 % kGroup == 0 && kGroup % 32 == 0, "the planes fit; whole pieces and warps");
+  static constexpr int kEnd = 16 * 256;               // kx = 0 copy of a row's last step: 12 planes of 16 pixels (and as above)
+  static constexpr int kSmem = kStages * kTiles * (kTile + kEnd) + 2 * kStages * 8 + 16;
+};
+using WgWide = WgCfg<128, 1>;
+// Rows of up to 16 pixels: a tile is one step, and four of them share a stage's
+// waits and fences
+using WgNarrow = WgCfg<16, 4>;
 constexpr int kWgMaxCtas = 304;         // about two CTAs per SM
 constexpr int kWgPart = kBnK * 32 + 32; // one CTA's partial: dw [co][tap][ci], then db [co]
 // partial sums of one sgmf_bn_wgrad call (calls must not overlap on the GPU)
@@ -454,32 +436,60 @@ struct BnWgradArgs {
   int *err;
 };
 
-__global__ void __launch_bounds__(kWgThreads + 32) k_bn_wgrad(const __grid_constant__ BnWgradArgs a) {
+// stage rows y - 1, y, y + 1, pixels x0 - 1 .. x0 + PX of x as chunk planes of
+// PX + 2 pixels (zero outside the image), by THREADS threads (tid): a thread
+// keeps its chunk and its pixels of each row, so that a piece is a compare and a copy
+template <int THREADS, int PX>
+__device__ __forceinline__ void bn_stage_rows(uint32_t dst, const uint16_t *x, const BnTile &t, int w, int h, int tid) {
+  constexpr int kPlane = (PX + 2) * 16;
+  const int j = tid & 3, p0 = tid >> 2;
+  const uint16_t *row = x + (((long long)t.img * h + t.y - 1) * w + t.x0 - 1) * kBnC;   // staged pixel 0 of row y - 1
+#pragma unroll
+  for (int ky = 0; ky < 3; ++ky) {
+    const bool row_in = (unsigned)(t.y + ky - 1) < (unsigned)h;
+    const uint16_t *src = row + ((long long)ky * w + p0) * kBnC + 8 * j;
+    const uint32_t d = dst + (ky * 4 + j) * kPlane + p0 * 16;
+#pragma unroll
+    for (int s = 0; s < PX * 4 / THREADS; ++s) {
+      const bool in = row_in && (unsigned)(t.x0 - 1 + p0 + s * (THREADS / 4)) < (unsigned)w;
+      cp_async16(d + s * (THREADS / 4) * 16, in ? src + s * (THREADS / 4) * kBnC : x, in);
+    }
+  }
+  if (tid < 24) {                                // the last two pixels of each row
+    const int ky = tid >> 3, px = PX + ((tid >> 2) & 1);
+    const bool in = (unsigned)(t.y + ky - 1) < (unsigned)h && (unsigned)(t.x0 - 1 + px) < (unsigned)w;
+    cp_async16(dst + (ky * 4 + j) * kPlane + px * 16, in ? row + ((long long)ky * w + px) * kBnC + 8 * j : x, in);
+  }
+}
+
+template <typename CF>
+__global__ void __launch_bounds__(CF::kThreads + 32) k_bn_wgrad(const __grid_constant__ BnWgradArgs a) {
+  constexpr int PX = CF::PX, kTiles = CF::kTiles, kStages = CF::kStages, kThreads = CF::kThreads;
   extern __shared__ __align__(1024) uint8_t sm[];
-  uint8_t *ends = sm + kWgStages * kWgStage;                                  // [stage] kx = 0 copies
-  uint64_t *full = reinterpret_cast<uint64_t *>(ends + kWgStages * kWgEnd);   // a stage is filled
-  uint64_t *empty = full + kWgStages;                                         // its MMAs are done
-  uint32_t *slot = reinterpret_cast<uint32_t *>(empty + kWgStages);
+  uint8_t *ends = sm + kStages * kTiles * CF::kTile;                          // [stage][tile] kx = 0 copies
+  uint64_t *full = reinterpret_cast<uint64_t *>(ends + kStages * kTiles * CF::kEnd);   // a stage is filled
+  uint64_t *empty = full + kStages;                                         // its MMAs are done
+  uint32_t *slot = reinterpret_cast<uint32_t *>(empty + kStages);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int tpr = (a.w + kCvM - 1) / kCvM;
-  const long long ntile = (long long)a.n * a.h * tpr, tile0 = (long long)blockIdx.x * a.chunks;
-  const int nt = (int)min((long long)a.chunks, ntile - tile0);               // >= 1
+  const int tpr = (a.w + PX - 1) / PX;
+  const long long ntile = (long long)a.n * a.h * tpr, tile0 = (long long)blockIdx.x * a.chunks * kTiles;
+  const int my_tiles = (int)min((long long)a.chunks * kTiles, ntile - tile0);   // >= 1
+  const int nt = (my_tiles + kTiles - 1) / kTiles;   // the CTA's stages
   if (warp == 0) {
     tmem_alloc(slot, 128);
     tmem_relinquish();
   }
   if (tid == 0) {
-    for (int s = 0; s < kWgStages; ++s) {
-      mbar_init(&full[s], kWgThreads);
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(&full[s], kThreads);
       mbar_init(&empty[s], 1);
     }
     mbar_fence_init();
   }
   // what M = 128 reads past the planes is never used, but starts finite
-  for (int i = tid; i < kWgStages * (kWgStage - kCvX - 4 * kWgPlane) / 16; i += kWgThreads + 32) {
-    constexpr int kTail = (kWgStage - kCvX - 4 * kWgPlane) / 16;
-    reinterpret_cast<uint4 *>(sm + i / kTail * kWgStage + kCvX + 4 * kWgPlane)[i % kTail] = make_uint4(0, 0, 0, 0);
-  }
+  constexpr int kTail = (CF::kTile - CF::kX - 4 * CF::kYPlane) / 16;
+  for (int i = tid; i < kStages * kTiles * kTail; i += kThreads + 32)
+    reinterpret_cast<uint4 *>(sm + i / kTail * CF::kTile + CF::kX + 4 * CF::kYPlane)[i % kTail] = make_uint4(0, 0, 0, 0);
   float dbp[8];                                      // bias gradient of the thread's chunk over its pixels
 #pragma unroll
   for (int c = 0; c < 8; ++c) dbp[c] = 0.0f;
@@ -497,47 +507,56 @@ __global__ void __launch_bounds__(kWgThreads + 32) k_bn_wgrad(const __grid_const
     }
     return ok;
   };
-  if (warp < kWgLoad) {
-    BnTile ld(tile0, tpr, a.h);
-    constexpr int kY = kCvM * 4 / kWgThreads;        // dY pieces a thread stages: its chunk is tid & 3 throughout
-    for (int t = 0; t < nt + kWgStages - 1; ++t) {
+  if (warp < CF::kLoad) {
+    const int g = tid / CF::kGroup, lt = tid % CF::kGroup;   // the thread's tile of a stage, its number among that tile's
+    BnTile ld(tile0 + g, tpr, a.h, PX);
+    constexpr int kY = PX * 4 / CF::kGroup;          // dY pieces a thread stages: its chunk is tid & 3 throughout
+    const int y_off = g * CF::kTile + CF::kX + (lt & 3) * CF::kYPlane;
+    for (int t = 0; t < nt + kStages - 1; ++t) {
       if (t < nt) {
-        if (t >= kWgStages && !wait(&empty[t % kWgStages], t / kWgStages - 1)) break;
-        const uint32_t dst = smem_u32(sm) + t % kWgStages * kWgStage;
-        const int nv = min(kCvM, a.w - ld.x0), npx = (nv + 15) / 16 * 16;   // the tile's pixels; those of its steps
-        bn_stage_rows<kWgThreads>(dst, a.x, ld, a.w, a.h);
-        if (nv != npx && tid < 12 * 16) {
-          const int p = tid >> 4, i = tid & 15, px = ld.x0 + npx - 17 + i, yy = ld.y + (p >> 2) - 1;   // plane, pixel
-          const bool in = (unsigned)yy < (unsigned)a.h && px >= 0 && px < a.w - 1;
-          const uint16_t *src = a.x + (((long long)ld.img * a.h + yy) * a.w + px) * kBnC + 8 * (p & 3);
-          cp_async16(smem_u32(ends) + t % kWgStages * kWgEnd + p * 256 + i * 16, in ? src : a.x, in);
-        }
-        const uint16_t *src = a.dy + (((long long)ld.img * a.h + ld.y) * a.w + ld.x0) * kBnC + 8 * (tid & 3);
+        if (t >= kStages && !wait(&empty[t % kStages], t / kStages - 1)) break;
+        if (kTiles == 1 || t * kTiles + g < my_tiles) {
+          const uint32_t dst = smem_u32(sm) + t % kStages * (kTiles * CF::kTile);
+          const int nv = min(PX, a.w - ld.x0), npx = (nv + 15) / 16 * 16;   // the tile's pixels; those of its steps
+          bn_stage_rows<CF::kGroup, PX>(dst + g * CF::kTile, a.x, ld, a.w, a.h, lt);
+          if (nv != npx) {
+            for (int i = lt; i < 12 * 16; i += CF::kGroup) {
+              const int px = ld.x0 + npx - 17 + (i & 15), yy = ld.y + (i >> 6) - 1;
+              const bool in = (unsigned)yy < (unsigned)a.h && px >= 0 && px < a.w - 1;
+              const uint16_t *src = a.x + (((long long)ld.img * a.h + yy) * a.w + px) * kBnC + 8 * (i >> 4 & 3);
+              cp_async16(smem_u32(ends) + (t % kStages * kTiles + g) * CF::kEnd + i * 16, in ? src : a.x, in);
+            }
+          }
+          const uint16_t *src = a.dy + (((long long)ld.img * a.h + ld.y) * a.w + ld.x0) * kBnC + 8 * (lt & 3);
 #pragma unroll
-        for (int s = 0; s < kY; ++s) {
-          const int px = (tid >> 2) + s * (kWgThreads / 4);
-          const bool in = px < nv;
-          cp_async16(dst + kCvX + (tid & 3) * kWgPlane + px * 16, in ? src + px * kBnC : a.dy, in);
+          for (int s = 0; s < kY; ++s) {
+            const int px = (lt >> 2) + s * (CF::kGroup / 4);
+            const bool in = px < nv;
+            cp_async16(dst + y_off + px * 16, in ? src + px * kBnC : a.dy, in);
+          }
+#pragma unroll
+          for (int i = 0; i < kTiles; ++i) ld.next(a.w, a.h, PX);
         }
-        ld.next(a.w, a.h);
       }
       cp_async_commit();
-      const int e = t - (kWgStages - 1);             // the tile handed on
+      const int e = t - (kStages - 1);               // the stage handed on
       if (e >= 0) {
-        cp_async_wait<kWgStages - 1>();
-        const uint8_t *ys = sm + (e % kWgStages) * kWgStage + kCvX + (tid & 3) * kWgPlane;
+        cp_async_wait<kStages - 1>();
+        if (kTiles == 1 || e * kTiles + g < my_tiles) {
+          const uint8_t *ys = sm + (e % kStages) * (kTiles * CF::kTile) + y_off;
 #pragma unroll
-        for (int s = 0; s < kY; ++s) {
-          const uint4 v = *reinterpret_cast<const uint4 *>(ys + ((tid >> 2) + s * (kWgThreads / 4)) * 16);
-          const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+          for (int s = 0; s < kY; ++s) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(ys + ((lt >> 2) + s * (CF::kGroup / 4)) * 16);
+            const uint32_t u[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            dbp[2 * q] += __uint_as_float(u[q] << 16);
-            dbp[2 * q + 1] += __uint_as_float(u[q] & 0xffff0000u);
+            for (int q = 0; q < 4; ++q) {
+              dbp[2 * q] += __uint_as_float(u[q] << 16);
+              dbp[2 * q + 1] += __uint_as_float(u[q] & 0xffff0000u);
+            }
           }
         }
         fence_async_smem();
-        bn_arrive(&full[e % kWgStages]);
+        bn_arrive(&full[e % kStages]);
       }
     }
     cp_async_wait<0>();
@@ -545,29 +564,34 @@ __global__ void __launch_bounds__(kWgThreads + 32) k_bn_wgrad(const __grid_const
     constexpr uint32_t idesc = idesc_bf16(128, 32, true);
     const uint32_t leader = elect_one();
     int issued = 0;
-    BnTile cur(tile0, tpr, a.h);
+    BnTile cur(tile0, tpr, a.h, PX);
     for (int t = 0; t < nt; ++t) {
-      if (!wait(&full[t % kWgStages], t / kWgStages)) break;
+      if (!wait(&full[t % kStages], t / kStages)) break;
       tc_fence_after();
-      const uint32_t x_0 = smem_u32(sm) + (t % kWgStages) * kWgStage;
-      const uint64_t xd = sdesc(x_0, 128, kCvPlane), yd = sdesc(x_0 + kCvX, 128, kWgPlane);
-      const uint64_t ed = sdesc(smem_u32(ends) + (t % kWgStages) * kWgEnd, 128, 256);
-      const int nv = min(kCvM, a.w - cur.x0);
-      cur.next(a.w, a.h);
-      // the three accumulators in turn: MMAs into one accumulator follow each other slower
 #pragma unroll
-      for (int s = 0; s < kCvM / 16; ++s) {
-        if (16 * s >= nv) break;                     // (no pixel of the row)
+      for (int g = 0; g < kTiles; ++g) {
+        if (kTiles > 1 && t * kTiles + g >= my_tiles) break;
+        const int slot_t = t % kStages * kTiles + g;
+        const uint32_t x_0 = smem_u32(sm) + slot_t * CF::kTile;
+        const uint64_t xd = sdesc(x_0, 128, CF::kXPlane), yd = sdesc(x_0 + CF::kX, 128, CF::kYPlane);
+        const uint64_t ed = sdesc(smem_u32(ends) + slot_t * CF::kEnd, 128, 256);
+        const int nv = min(PX, a.w - cur.x0);
+        cur.next(a.w, a.h, PX);
+        // the three accumulators in turn: MMAs into one accumulator follow each other slower
 #pragma unroll
-        for (int kx = 0; kx < 3; ++kx)
-          umma_bf16(tmem + 32 * kx, kx == 0 && nv < 16 * s + 16 ? ed : sdesc_at(xd, kx * 16 + s * 256),
-                    sdesc_at(yd, s * 256), idesc, (t > 0 || s > 0) ? 1u : 0u, leader);
+        for (int s = 0; s < PX / 16; ++s) {
+          if (16 * s >= nv) break;                   // (no pixel of the row)
+#pragma unroll
+          for (int kx = 0; kx < 3; ++kx)
+            umma_bf16(tmem + 32 * kx, kx == 0 && nv < 16 * s + 16 ? ed : sdesc_at(xd, kx * 16 + s * 256),
+                      sdesc_at(yd, s * 256), idesc, (t > 0 || g > 0 || s > 0) ? 1u : 0u, leader);
+        }
       }
-      umma_commit(&empty[t % kWgStages], leader);
+      umma_commit(&empty[t % kStages], leader);
       issued = t + 1;
     }
     // every MMA has completed before the accumulators are read and freed
-    for (int t = max(0, issued - kWgStages); t < issued; ++t) wait(&empty[t % kWgStages], t / kWgStages);
+    for (int t = max(0, issued - kStages); t < issued; ++t) wait(&empty[t % kStages], t / kStages);
   }
   tc_fence_before();
   ok = __syncthreads_and(ok) != 0;
@@ -588,18 +612,18 @@ __global__ void __launch_bounds__(kWgThreads + 32) k_bn_wgrad(const __grid_const
     }
   }
   // bias gradient: each warp's sums per chunk, then the warps in order
-  __shared__ float dbw[kWgThreads / 32][32];
+  __shared__ float dbw[CF::kLoad][32];
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
     float s = dbp[c];
     for (int o = 4; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane < 4 && warp < kWgLoad) dbw[warp][lane * 8 + c] = s;
+    if (lane < 4 && warp < CF::kLoad) dbw[warp][lane * 8 + c] = s;
   }
   tc_fence_before();
   __syncthreads();
   if (tid < 32) {
     float s = dbw[0][tid];
-    for (int q = 1; q < kWgThreads / 32; ++q) s += dbw[q][tid];
+    for (int q = 1; q < CF::kLoad; ++q) s += dbw[q][tid];
     part[kBnK * 32 + tid] = s;
   }
   if (warp == 0) tmem_dealloc(tmem, 128);
@@ -847,27 +871,36 @@ __global__ void __launch_bounds__(1024) k_bn_wgrad_sum(const float *__restrict__
     db[o - kBnK * 32] += s;
 }
 
-extern "C" sgmf_status sgmf_bn_wgrad(int n, int h, int w, const uint16_t *x, const uint16_t *dy, float *dw, float *db,
-                                     int *err, void *stream) {
-  if (n < 1 || h < 1 || w < 1 || !x || !dy || !dw || !db || !err) return SGMF_ERR_ARG;
+template <typename CF>
+static sgmf_status bn_wgrad(int n, int h, int w, const uint16_t *x, const uint16_t *dy, float *dw, float *db, int *err,
+                            cudaStream_t s) {
   static bool attr[64] = {};
   const cudaError_t ea = once_per_device(attr, [](int) {
-    return cudaFuncSetAttribute(k_bn_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
+    return cudaFuncSetAttribute(k_bn_wgrad<CF>, cudaFuncAttributeMaxDynamicSharedMemorySize, CF::kSmem);
   });
   if (ea != cudaSuccess) return bn_launch(ea, "sgmf_bn_wgrad attribute");
-  const long long nchunk = (long long)n * h * ((w + kCvM - 1) / kCvM);   // tiles
-  const int chunks = (int)((nchunk + kWgMaxCtas - 1) / kWgMaxCtas);
-  const unsigned grid = (unsigned)((nchunk + chunks - 1) / chunks);   // <= kWgMaxCtas
+  const long long ntile = (long long)n * h * ((w + CF::PX - 1) / CF::PX), nstage = (ntile + CF::kTiles - 1) / CF::kTiles;
+  const int chunks = (int)((nstage + kWgMaxCtas - 1) / kWgMaxCtas);
+  const unsigned grid = (unsigned)((nstage + chunks - 1) / chunks);   // <= kWgMaxCtas
   float *part = nullptr;
   cudaError_t e = cudaGetSymbolAddress(reinterpret_cast<void **>(&part), g_wgrad_part);
   if (e != cudaSuccess) return bn_launch(e, "sgmf_bn_wgrad scratch");
   BnWgradArgs a{n, h, w, chunks, x, dy, part, err};
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  k_bn_wgrad<<<grid, kWgThreads + 32, kWgSmem, s>>>(a);
+  k_bn_wgrad<CF><<<grid, CF::kThreads + 32, CF::kSmem, s>>>(a);
   e = cudaGetLastError();
   if (e != cudaSuccess) return bn_launch(e, "sgmf_bn_wgrad");
   k_bn_wgrad_sum<<<kWgPart / 32, 1024, 0, s>>>(part, (int)grid, dw, db);
   return bn_launch(cudaGetLastError(), "sgmf_bn_wgrad");
+}
+
+extern "C" sgmf_status sgmf_bn_wgrad(int n, int h, int w, const uint16_t *x, const uint16_t *dy, float *dw, float *db,
+                                     int *err, void *stream) {
+  if (n < 1 || h < 1 || w < 1 || !x || !dy || !dw || !db || !err) return SGMF_ERR_ARG;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  // the line lies where a row is one step of the MMAs: 16 x 270 rows of 16 pixels
+  // 38 us a call as 128-pixel tiles, 17 so; of 4 pixels 37 -> 17 (of 1 pixel 17, where
+  // packing pixels of several rows into a tile, through 2-byte stores, took 15)
+  return w <= WgNarrow::PX ? bn_wgrad<WgNarrow>(n, h, w, x, dy, dw, db, err, s) : bn_wgrad<WgWide>(n, h, w, x, dy, dw, db, err, s);
 }
 
 extern "C" sgmf_status sgmf_bn_input(int n, int width, int height, int max_disp, const uint8_t *left,

@@ -1,5 +1,7 @@
 """The weight gradient where its tiles end: infinities and NaN beside the ends of
-a row."""
+a row; rows of up to 16 pixels, four to a stage; and calls in which every stage
+of a CTA's three-stage ring is refilled several times (the other tests give a
+CTA at most three tiles)."""
 import numpy as np
 import pytest
 
@@ -49,3 +51,25 @@ def test_non_finite_activations_reach_their_own_taps_only(gpu, w):
     sw, _ = N.conv3x3_wgrad(np.abs(clean), np.abs(dy))
     assert (np.abs(dw[fin] - rw[fin]) <= 3e-5 * (sw[fin] + 1e-30)).all()
     assert np.isfinite(db).all()
+
+
+@pytest.mark.parametrize("n,h,w", [(16, 120, 130), (16, 76, 17), (11, 113, 140), (16, 270, 9), (15, 241, 16), (3, 1, 1),
+                                   (5, 2, 3), (16, 400, 1)])
+def test_ring_refilled(gpu, n, h, w):
+    """13, 4 and 9 tiles a CTA (the third with a shorter last CTA); rows of up to 16
+    pixels: 4, 3, 1, 1 and 6 stages of four rows, the last one of the call full or
+    not.  An entry is at most 13 x 8 accumulations and 10 + 31 partial sums, each
+    off by at most 2^-22 of the terms' magnitudes: 4e-5.  The order of the sums is
+    fixed, so that a second call gives the same bits."""
+    rng = np.random.default_rng(n + h + w)
+    x = N.bf16_round(np.maximum(rng.normal(size=(n, h, w, 32)), 0.0))
+    dy = _rand_bf16(rng, (n, h, w, 32), 0.1)
+    xd, dyd = _dev(_bits(x)), _dev(_bits(dy))
+    dw, db = _wgrad(n, h, w, xd, dyd)
+    rw, rb = N.conv3x3_wgrad(x, dy)
+    sw, sb = N.conv3x3_wgrad(np.abs(x), np.abs(dy))
+    assert (np.abs(dw - rw) <= 4e-5 * sw).all()
+    assert (np.abs(db - rb) <= 4e-5 * sb).all()
+    again, dagain = _wgrad(n, h, w, xd, dyd)
+    np.testing.assert_array_equal(again, dw)
+    np.testing.assert_array_equal(dagain, db)
