@@ -452,8 +452,8 @@ extern "C" int sgmf_launches_per_compute(const sgmf_ctx *c) {
   if (!c) return 0;
   // front stages, then the sweep, rows and check (once per part of a batch in
   // parts; counted for a full batch), or one launch per line family, the rows
-  // among them (two where their costs are u16), and the winner kernel, which checks
-  const int agg = use_sweep(c) ? 3 : (c->k.num_paths == 8 ? 3 : 1) + (c->spill8 ? 1 : 2) + 1;
+  // among them, and the winner kernel, which checks
+  const int agg = use_sweep(c) ? 3 : (c->k.num_paths == 8 ? 4 : 2) + 1;
   int parts = 1;
   if (use_sweep(c) && sweep_part(c, c->nb) > 0) {
     const int m = sweep_part(c, c->nb);
@@ -545,11 +545,15 @@ static sgmf_status front_stages(sgmf_ctx *c, int f0, int nf, const uint8_t *left
 // 647 us, of 640 x 120, D = 128 (6.3) 485 -> 486, of 1242 x 200, D = 128 (10.5)
 // 1529 -> 1213.  Above 12 rows a SM it depends on the shape, and the row kernel
 // stays: 13 frames of 1242 x 375 2907 against 2978 us, 12 of 320 x 240, D = 64 474
-// against 490, though 12 of 640 x 480, D = 64 1360 against 1277.
-constexpr int kRowLinesPerSm = 12;
+// against 490, though 12 of 640 x 480, D = 64 1360 against 1277.  With u16 costs
+// the winner kernel steps every second column itself, and the rows have to be
+// long as well: 8 frames of 1332 x 53, D = 124 1104 -> 633 us, of 1000 x 180, D =
+// 128 1065 -> 1015, of 700 x 100, D = 64 351 -> 332, but of 640 x 120, D = 128 485
+// -> 495 and of 500 x 100, D = 192 706 -> 755.
+constexpr int kRowLinesPerSm = 12, kRowLinesU16 = 700;
 static bool rows_as_lines(const sgmf_ctx *c, int nf) {
   int sms = 0;
-  if (!c->spill8 || sm_count(&sms) != cudaSuccess) return false;
+  if (sm_count(&sms) != cudaSuccess || (!c->spill8 && c->k.W < kRowLinesU16)) return false;
   return (long)c->k.H * nf <= (long)kRowLinesPerSm * sms;
 }
 
@@ -569,18 +573,26 @@ static sgmf_status finish(sgmf_ctx *c, KParams ka, const Buffers &b, int nf, int
 }
 
 // Whether the line walks of a call of n frames store the vectors of every
-// second row (column) only and the winner kernel takes the others' steps: 17
-// instead of 24 bytes a cell through memory for about half as many instructions
-// again in the winner kernel.  It pays where the volumes are far larger than the
-// L2 (1242 x 375, D = 128: one frame of 60 M cells 377 -> 397 us, two 651 -> 616,
-// eight 2100 -> 1943; four paths, half the walks to save on: 119 M cells 416 ->
-// 425, 238 M 646 -> 628) and where a lane's 16 or 24 cells spread the steps'
-// fixed work without filling the registers: at Dp = 64 640 x 480 x 12 1411 ->
-// 1504 us, at Dp = 256 1920 x 1080 x 4 8550 -> 10460.
+// second row (of the rows: column) only and the winner kernel takes the others'
+// steps.
+// Bytes: 17 instead of 24 bytes a cell through memory for about half as many
+// instructions again in the winner kernel.  It pays where the volumes are far
+// larger than the L2 (1242 x 375, D = 128: one frame of 60 M cells 377 -> 397 us,
+// two 651 -> 616, eight 2100 -> 1943; four paths, half the walks to save on: 119 M
+// cells 416 -> 425, 238 M 646 -> 628) and where a lane's 16 or 24 cells spread
+// the steps' fixed work without filling the registers: at Dp = 64 640 x 480 x 12
+// 1411 -> 1504 us, at Dp = 256 1920 x 1080 x 4 8550 -> 10460.
+// u16: the rows' vectors are half stored in any case (they share a region); the
+// other families' for 25 instead of 37 bytes a cell, earlier and at every width: 640 x
+// 480, D = 64 20 M cells 200 -> 228 us, 39 M 333 -> 336, 79 M 697 -> 565; 333 x 217,
+// D = 100 9 M 143 -> 150, 28 M 240 -> 216; 1920 x 1080 x 4, D = 256 12443 -> 10092.
+// Four paths: 28 M cells 162 -> 169, 60 M 317 -> 308, 123 M 551 -> 504.  Bands of
+// 64: 59 M 622 -> 654, 79 M 642 -> 620, 133 M 1208 -> 1222, 531 M 3969 -> 3756.
 static int half_vectors(const sgmf_ctx *c, int n) {
   const KParams &k = c->k;
-  return c->spill8 && !k.band && (k.Dp == 128 || k.Dp == 192) &&
-         frame_cells(k) * n >= (k.num_paths == 8 ? 100000000u : 200000000u);
+  const size_t cells = frame_cells(k) * n;
+  if (!c->spill8) return cells >= (k.band ? 100000000u : (k.num_paths == 8 ? 25000000u : 50000000u));
+  return !k.band && (k.Dp == 128 || k.Dp == 192) && cells >= (k.num_paths == 8 ? 100000000u : 200000000u);
 }
 
 // Aggregation, winners and check of the n frames whose cost volume is made.

@@ -11,7 +11,8 @@
 //   path costs      2 Dp bytes a pixel and line family (vertical, two diagonals): both
 //                                           directions' byte vectors, u16 vectors of one,
 //                                           or (the first two) the sweep's u16 sums
-//   spill           4 such regions: the rows' path costs, u16 vectors of the other directions
+//   spill           4 such regions: the rows' path costs (u16: every second column's of both
+//                                           directions), u16 vectors of the other directions
 // F is the number of frames a context holds (its batch capacity); every
 // kernel takes the frame from its last grid dimension.
 #pragma once

@@ -224,6 +224,12 @@ __device__ __forceinline__ void pad_bytes(int D, int lig, uint32_t (&z)[CPL / 4]
 }
 
 
+template <int NW>
+__device__ __forceinline__ void copy_words(uint32_t (&dst)[NW], const uint32_t (&src)[NW]) {
+#pragma unroll
+  for (int w = 0; w < NW; ++w) dst[w] = src[w];
+}
+
 struct StepConsts {
   uint32_t p1x2;   // P1 in both halves
   uint32_t dpx2;   // (P2 - P1) in both halves

@@ -37,7 +37,6 @@ struct LineArgs {
   size_t dst_frame[2];    // bytes from one frame to the next
   StepConsts sc;
   const int *gate;        // per-frame gate words of the launch's frames, or null
-  int dir;                // the direction of a launch of one direction
   const int16_t *lo;      // banded mode: band starts per tile, [frame][th][tw]
 };
 
@@ -63,13 +62,14 @@ struct LinePos {
 constexpr int kLineAhead = 16;   // steps copied ahead (a multiple of the four unrolled)
 
 // HALF: store only the vectors of even rows (rows family: even columns); the
-// winner kernel takes the others' step itself.
-// ADD: the vector of the pixel's other direction, there already, is added (u16
-// rows: one vector for both).  BANDED: on the bands (no padding cells).
-template <int CPL, bool S8, int FAM, bool BANDED, bool ADD, bool HALF>
+// winner kernel takes the others' step itself.  With u16 vectors the two
+// directions of the rows then share a region: that of left -> right in its
+// pixel's place, that of right -> left in the place of the pixel before, column
+// 0's in its own (the other one there is the cost itself).
+// BANDED: on the bands (no padding cells).
+template <int CPL, bool S8, int FAM, bool BANDED, bool HALF>
 __global__ void __launch_bounds__(256) k_lines(const __grid_constant__ LineArgs a) {
-  constexpr int NW = CPL / 2, Dp = kGL * CPL, A = kLineAhead, U = 4, k8 = 32 * CPL, kSlot = k8 * (ADD ? 3 : 1);
-  static_assert(!(ADD && S8), "byte vectors have a place each");
+  constexpr int NW = CPL / 2, Dp = kGL * CPL, A = kLineAhead, U = 4, kSlot = 32 * CPL;
   extern __shared__ __align__(128) uint8_t smem[];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int f = blockIdx.z;
@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(256) k_lines(const __grid_constant__ LineArgs 
     asm volatile("griddepcontrol.wait;" ::: "memory");
     return;
   }
-  const bool up = gridDim.y == 1 ? a.dir != 0 : blockIdx.y != 0;
+  const bool up = blockIdx.y != 0;
   const int line = min(line0 + grp, lines - 1);  // a group past the last line repeats it and stores nothing
   const bool act = line0 + grp < lines;
   const uint8_t *cost = a.cost + f * frame_cells(a.k) + lig * Vec8<CPL>::kLane;
@@ -117,7 +117,6 @@ __global__ void __launch_bounds__(256) k_lines(const __grid_constant__ LineArgs 
   LinePos<FAM> at = in;                          // in: next step to copy; at: next step to take
   auto copy = [&](uint32_t slot) {
     copy8<CPL>(slot, lane, cost + (size_t)(unsigned)in.p * Dp);
-    if constexpr (ADD) copy16<CPL>(slot + k8, lane, dst + (size_t)(unsigned)in.p * (2 * Dp));
     in.next(dp, dx, dy, xw, xs, W);
   };
 #pragma unroll 1
@@ -145,11 +144,9 @@ __global__ void __launch_bounds__(256) k_lines(const __grid_constant__ LineArgs 
   slot_raw8<CPL>(ring, lane, nxt);
   // a step on the bytes read before; slot: the next step's.  The copy into
   // the slot of the step itself follows (its bytes are in registers)
-  auto take = [&](const uint8_t *slot, [[maybe_unused]] const uint8_t *own) {
+  auto take = [&](const uint8_t *slot) {
     uint32_t C[NW];
     expand8<CPL>(nxt, z, C);
-    [[maybe_unused]] uint32_t other[NW];
-    if constexpr (ADD) slot16<CPL>(own + k8, lane, other);
     cp_wait<A - 2>();
     slot_raw8<CPL>(slot, lane, nxt);
     Edges e = none;
@@ -173,10 +170,8 @@ __global__ void __launch_bounds__(256) k_lines(const __grid_constant__ LineArgs 
     step<NW, BANDED>(L, C, mm, sc, e, lig);
     mm = group_min<NW>(L);
     uint8_t *o = dst + (size_t)(unsigned)at.p * (2 * Dp);
-    if constexpr (ADD) {
-#pragma unroll
-      for (int w = 0; w < NW; ++w) other[w] += L[w];
-      if (act) store_u16<CPL>(o, other);
+    if constexpr (HALF && FAM == 3 && !S8) {
+      if (act && !(at.x & 1) && (up || at.x != 0)) VecW<CPL, S8>::put(up && at.x != 0 ? o - 2 * Dp : o, L);
     } else if (act && !(HALF && ((FAM == 3 ? at.x : at.y) & 1))) {
       VecW<CPL, S8>::put(o, L);
     }
@@ -187,7 +182,7 @@ __global__ void __launch_bounds__(256) k_lines(const __grid_constant__ LineArgs 
     const int after = base + U * kSlot == A * kSlot ? 0 : base + U * kSlot;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      take(ring + (u + 1 < U ? base + (u + 1) * kSlot : after), ring + base + u * kSlot);
+      take(ring + (u + 1 < U ? base + (u + 1) * kSlot : after));
       copy(ring_s + base + u * kSlot);
       cp_commit();
     }
@@ -196,7 +191,7 @@ __global__ void __launch_bounds__(256) k_lines(const __grid_constant__ LineArgs 
 #pragma unroll 1
   for (; t < n; ++t) {
     const int after = base + kSlot == A * kSlot ? 0 : base + kSlot;
-    take(ring + after, ring + base);             // (past the last step: bytes never used)
+    take(ring + after);                          // (past the last step: bytes never used)
     if (t + A < n) copy(ring_s + base);
     cp_commit();
     base = after;
@@ -207,17 +202,18 @@ __global__ void __launch_bounds__(256) k_lines(const __grid_constant__ LineArgs 
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-template <int CPL, bool S8, int FAM, bool BANDED, bool ADD = false, bool HALF = false>
-static cudaError_t launch_family(const LineArgs &a, int nf, int dirs, bool overlap, cudaStream_t s) {
-  constexpr int kWarp = kLineAhead * 32 * CPL * (ADD ? 3 : 1) + (BANDED ? kGW * kGL * CPL * 2 : 0);
-  constexpr int kFit = 224 * 1024 / kWarp, kMaxWarps = kFit < 8 ? kFit : 8;   // (the ADD walks' rings are three times as long)
+template <int CPL, bool S8, int FAM, bool BANDED, bool HALF>
+static cudaError_t launch_family(const LineArgs &a, int nf, bool overlap, cudaStream_t s) {
+  constexpr int kWarp = kLineAhead * 32 * CPL + (BANDED ? kGW * kGL * CPL * 2 : 0);
+  constexpr int kMaxWarps = 8;
+  static_assert(kMaxWarps * kWarp <= 224 * 1024, "the rings fit");
   const int warps = std::min(a.k.line_warps, kMaxWarps), per_cta = kGW * warps, lines = FAM == 3 ? a.k.H : a.k.W;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((lines + per_cta - 1) / per_cta, dirs, nf);
+  cfg.gridDim = dim3((lines + per_cta - 1) / per_cta, 2, nf);
   cfg.blockDim = dim3(32 * warps);
   cfg.dynamicSmemBytes = warps * kWarp;
   static bool done[64] = {};
-  const cudaError_t e = smem_optin(k_lines<CPL, S8, FAM, BANDED, ADD, HALF>, kMaxWarps * kWarp, done);
+  const cudaError_t e = smem_optin(k_lines<CPL, S8, FAM, BANDED, HALF>, kMaxWarps * kWarp, done);
   if (e != cudaSuccess) return e;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -225,13 +221,13 @@ static cudaError_t launch_family(const LineArgs &a, int nf, int dirs, bool overl
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = overlap ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k_lines<CPL, S8, FAM, BANDED, ADD, HALF>, a);
+  return cudaLaunchKernelEx(&cfg, k_lines<CPL, S8, FAM, BANDED, HALF>, a);
 }
 
 // Where a family's down and up vectors of a pixel lie.  S8: side by side,
 // [down Dp bytes][up Dp bytes], in the family's buffer (rows: in the fourth
 // spill region); u16: the up vectors in the family's buffer, the down vectors
-// in the family's spill region, the rows' one sum in the fourth.
+// in the family's spill region, the rows' of both in the fourth (k_lines, HALF).
 inline void family_vectors(const KParams &k, const Buffers &b, bool s8, int fam, uint8_t *(&v)[2], size_t (&frame)[2]) {
   const size_t cells = frame_cells(k);
   uint8_t *region = static_cast<uint8_t *>(b.spill) + fam * 2 * cells;
@@ -258,26 +254,20 @@ static cudaError_t launch_walks(const KParams &k, const Buffers &b, int nf, cuda
   a.gate = b.gate;
   a.lo = b.band_lo;
   // the first launch waits for the cost volume as usual; the others may start
-  // beside it (they touch nothing it writes).  The rows, the longest walks, go
-  // first; with u16 costs their second direction adds to the first one's
-  // vectors: two launches, the second after everything before it
+  // beside it (they touch nothing it writes).  The rows, the longest walks, go first
   bool overlap = false;
   cudaError_t e = cudaSuccess;
   auto family = [&](auto fam) {
     constexpr int F = decltype(fam)::value;
     if (e != cudaSuccess) return;
     family_vectors(k, b, S8, F, a.dst, a.dst_frame);
-    if constexpr (F == 3 && !S8) {
-      a.dir = 0;
-      e = launch_family<CPL, S8, F, BANDED>(a, nf, 1, false, s);
-      a.dir = 1;
-      if (e == cudaSuccess) e = launch_family<CPL, S8, F, BANDED, true>(a, nf, 1, false, s);
-    } else if constexpr (S8 && !BANDED && (CPL == 16 || CPL == 24)) {
-      e = k.half ? launch_family<CPL, S8, F, BANDED, false, true>(a, nf, 2, overlap, s)
-                 : launch_family<CPL, S8, F, BANDED>(a, nf, 2, overlap, s);
-    } else {
-      e = launch_family<CPL, S8, F, BANDED>(a, nf, 2, overlap, s);
-    }
+    if constexpr (!S8 && F == 3)
+      e = launch_family<CPL, S8, F, BANDED, true>(a, nf, overlap, s);
+    else if constexpr (!S8 || (!BANDED && (CPL == 16 || CPL == 24)))
+      e = k.half ? launch_family<CPL, S8, F, BANDED, true>(a, nf, overlap, s)
+                 : launch_family<CPL, S8, F, BANDED, false>(a, nf, overlap, s);
+    else
+      e = launch_family<CPL, S8, F, BANDED, false>(a, nf, overlap, s);
     overlap = true;
   };
   family(std::integral_constant<int, 3>{});

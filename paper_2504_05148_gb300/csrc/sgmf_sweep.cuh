@@ -117,12 +117,6 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-template <int NW>
-__device__ __forceinline__ void copy_vec(uint32_t (&dst)[NW], const uint32_t (&src)[NW]) {
-#pragma unroll
-  for (int w = 0; w < NW; ++w) dst[w] = src[w];
-}
-
 template <int CPL>
 __global__ void __launch_bounds__(32 * SweepCfg<CPL>::kMaxWarps, 1) k_sweep(const __grid_constant__ SweepArgs a) {
   using CF = SweepCfg<CPL>;
@@ -235,7 +229,7 @@ __global__ void __launch_bounds__(32 * SweepCfg<CPL>::kMaxWarps, 1) k_sweep(cons
   // min follows, two vectors at a time (one pass of shuffles for both: 32 frames
   // of 1242 x 375, D = 128 3.08 -> 3.00 ms)
   auto move = [&](uint32_t(&o)[NW], const uint32_t(&pr)[NW], uint32_t mp, const uint32_t(&Cc)[NW]) {
-    copy_vec<NW>(o, pr);
+    copy_words<NW>(o, pr);
     step<NW, false, (NW < 8)>(o, Cc, mp, sc, none);
   };
   bool ok = true;
@@ -264,7 +258,7 @@ __global__ void __launch_bounds__(32 * SweepCfg<CPL>::kMaxWarps, 1) k_sweep(cons
     uint32_t eL[NW], eR[NW], meL, meR;
     {
       uint32_t pr[NW], mpr = mR[1];
-      copy_vec<NW>(pr, DR[1]);
+      copy_words<NW>(pr, DR[1]);
       if (!plain) {
         const uint32_t kr = xg + 1 < W ? 0xffffffffu : 0u;   // pixel 0's right predecessor inside
 #pragma unroll
@@ -314,28 +308,28 @@ __global__ void __launch_bounds__(32 * SweepCfg<CPL>::kMaxWarps, 1) k_sweep(cons
       minR &= kr;
     }
     uint32_t carry[NW], mcarry = mL[0];
-    copy_vec<NW>(carry, DL[0]);
+    copy_words<NW>(carry, DL[0]);
     move(DL[0], inL, minL, C0);
 #pragma unroll
     for (int i = 0; i < P; ++i) {
       uint32_t C[NW];
       if (i == 0)
-        copy_vec<NW>(C, C0);
+        copy_words<NW>(C, C0);
       else if (i == P - 1)
-        copy_vec<NW>(C, CP);
+        copy_words<NW>(C, CP);
       else
         load_u8<CPL>(st + i * Dp, z, C);
       move(V[i], V[i], mV[i], C);
       if (i >= 1 && i <= P - 2) {
         uint32_t nxt[NW];
         const uint32_t mnxt = mL[i];
-        copy_vec<NW>(nxt, DL[i]);
+        copy_words<NW>(nxt, DL[i]);
         move(DL[i], carry, mcarry, C);
         group_min2<NW>(V[i], DL[i], mV[i], mL[i]);
-        copy_vec<NW>(carry, nxt);
+        copy_words<NW>(carry, nxt);
         mcarry = mnxt;
         uint32_t pr[NW], mpr = mR[i + 1];
-        copy_vec<NW>(pr, DR[i + 1]);
+        copy_words<NW>(pr, DR[i + 1]);
         if (!plain) {
           const uint32_t ki = xg + i + 1 < W ? 0xffffffffu : 0u;
 #pragma unroll
@@ -346,10 +340,10 @@ __global__ void __launch_bounds__(32 * SweepCfg<CPL>::kMaxWarps, 1) k_sweep(cons
         if (i % 2 == 0) group_min2<NW>(DR[i - 1], DR[i], mR[i - 1], mR[i]);   // (i = 1 waits for i = 2)
       } else if (i == 0) {
         group_min2<NW>(V[0], DL[0], mV[0], mL[0]);
-        copy_vec<NW>(DR[0], eR);
+        copy_words<NW>(DR[0], eR);
         mR[0] = meR;
       } else {
-        copy_vec<NW>(DL[P - 1], eL);
+        copy_words<NW>(DL[P - 1], eL);
         mL[P - 1] = meL;
         move(DR[P - 1], inR, minR, C);
         group_min2<NW>(V[P - 1], DR[P - 1], mV[P - 1], mR[P - 1]);
