@@ -62,9 +62,43 @@ __global__ void __launch_bounds__(256) k_consistency(KParams k, Buffers b0, int1
   }
 }
 
+// A thread per pixel that takes both terms, in tiles of 32 columns by 8 rows:
+// where the list has nothing to gather or the call too few tiles of it
+__global__ void __launch_bounds__(256) k_consistency_px(KParams k, Buffers b0, int16_t *__restrict__ out) {
+  const int x = blockIdx.x * 32 + (threadIdx.x & 31), y = blockIdx.y * 8 + (threadIdx.x >> 5);
+  if (x >= k.W || y >= k.H) return;
+  const Buffers b = frame_view(k, b0, blockIdx.z);
+  if (gated_off(b.gate, k.gate_run)) return;
+  out += (size_t)blockIdx.z * frame_px(k);
+  const size_t p = (size_t)y * k.W + x;
+  const int ds = b.dstar[p], xm = x - ds;
+  const int dp = xm >= 0 && k.consistency != 2 && k.consistency != 3 ? (int)b.dprime[(size_t)y * k.W + xm] : -1;
+  const bool stereo_ok = dp >= 0 && abs(ds - dp) <= k.lr;
+  const bool lidar_ok = check_needs_lidar(k, stereo_ok) && check_lidar_term(k, b, x, y, ds);
+  check_store(k, b, out, p, ds, check_passes(k, stereo_ok, lidar_ok));
+}
+
+// The list costs a call its atomics, a barrier and a fourth of the CTAs: about 2
+// us where a window of few rows leaves nothing to win them back (one frame of 640 x
+// 480, r_c = 0 16.5 us a call by pixels, 18.7 with the list; r_c = 4 18.6, 20.7;
+// r_c = 8 19.4, 19.6; r_c = 80 41.3, 35.8; 8 frames of 320 x 240, 4 tiles a SM, r_c = 0
+// the kernel 10.2, 12.3, r_c = 6 16.4, 14.3), and where the LiDAR term alone
+// decides, every pixel is on it: one frame of 640 x 480, r_c = 20 20.7 us by pixels,
+// 24.8 with the list, 8 frames of 320 x 240 32.7, 28.6 for their shape.
+static bool by_pixel(const KParams &k, long tiles) {
+  const bool every = k.consistency == 2;           // every pixel is on the list
+  if (every && k.rc == 0) return true;
+  if (!every && (k.consistency != 0 || k.rc > 4)) return false;
+  int sms = 0;
+  return sm_count(&sms) == cudaSuccess && tiles < (k.rc <= 4 ? 5L : 4L) * sms;
+}
+
 cudaError_t launch_consistency(const KParams &k, const Buffers &b, int nf, int16_t *out, cudaStream_t s) {
-  dim3 grid((k.W + 31) / 32, (k.H + 8 * kRows - 1) / (8 * kRows), nf);
-  k_consistency<<<grid, 256, 0, s>>>(k, b, out);
+  const dim3 grid((k.W + 31) / 32, (k.H + 8 * kRows - 1) / (8 * kRows), nf);
+  if (by_pixel(k, (long)grid.x * grid.y * grid.z))
+    k_consistency_px<<<dim3(grid.x, (k.H + 7) / 8, nf), 256, 0, s>>>(k, b, out);
+  else
+    k_consistency<<<grid, 256, 0, s>>>(k, b, out);
   return cudaGetLastError();
 }
 
