@@ -5,6 +5,7 @@
 //   k_semidense   Eq. 5
 //   k_cost        Hamming cost + DDC, Eq. 4, materialised as uint8 [H][W][Dp]
 #include <cuda.h>
+#include <algorithm>
 #include <cstdint>
 
 #include "sgmf_cost.cuh"
@@ -324,11 +325,11 @@ int make_image_tmap(void *tmap_out, const uint8_t *base, int W, int H, int pitch
 // radius) 32 at a time: a ballot finds them, a shuffle hands out each one's
 // disparity, and every lane ORs its bit into the words of the radii that
 // reach it.  The work follows the number of valid pixels, not r.  The pixels of
-// kBoxChunks such steps are loaded at once, one load latency instead of three at
-// the default radius (32 frames of 1242 x 375, D = 128: both passes 312 -> 278 us).
-constexpr int kBoxChunks = 3;
-
-template <int MW>
+// CHUNKS such steps are loaded at once: three, one load latency instead of three at
+// the default radius (32 frames of 1242 x 375, D = 128: both passes 312 -> 278 us),
+// or one where both radii are 0 and a step holds the window (one frame, alone
+// with the check 20.7 -> 18.7 us a call).
+template <int MW, int CHUNKS>
 __global__ void __launch_bounds__(256) k_boxor_rows(const int16_t *__restrict__ disp, uint32_t *__restrict__ tmpS,
                                                    uint32_t *__restrict__ tmpC, int W, int H, int D, int rs,
                                                    int rc, const int *gate, int run) {
@@ -344,15 +345,15 @@ __global__ void __launch_bounds__(256) k_boxor_rows(const int16_t *__restrict__ 
 #pragma unroll
   for (int w = 0; w < MW; ++w) aS[w] = aC[w] = 0u;
   const int end = x0 + 31 + R;                 // the last pixel of any lane's window
-  for (int base = x0 - R; base <= end; base += 32 * kBoxChunks) {
-    int d[kBoxChunks];
+  for (int base = x0 - R; base <= end; base += 32 * CHUNKS) {
+    int d[CHUNKS];
 #pragma unroll
-    for (int c = 0; c < kBoxChunks; ++c) {
+    for (int c = 0; c < CHUNKS; ++c) {
       const int xs = base + 32 * c + lane;
       d[c] = (xs >= 0 && xs < W && xs <= end) ? (int)row[xs] : -1;
     }
 #pragma unroll
-    for (int c = 0; c < kBoxChunks; ++c) {
+    for (int c = 0; c < CHUNKS; ++c) {
       const int b0 = base + 32 * c;
       unsigned m = __ballot_sync(0xffffffffu, d[c] >= 0 && d[c] < D);
       while (m != 0u) {
@@ -529,7 +530,10 @@ template <int MW>
 static void launch_boxor_rows(const KParams &k, int nf, const int16_t *disp, uint32_t *tS, uint32_t *tC, int rs,
                               int rc, cudaStream_t s, const int *gate) {
   dim3 g((k.W + 31) / 32, (k.H + 7) / 8, nf);
-  k_boxor_rows<MW><<<g, 256, 0, s>>>(disp, tS, tC, k.W, k.H, k.D, rs, rc, gate, k.gate_run);
+  if (std::max(rs, rc) == 0)
+    k_boxor_rows<MW, 1><<<g, 256, 0, s>>>(disp, tS, tC, k.W, k.H, k.D, rs, rc, gate, k.gate_run);
+  else
+    k_boxor_rows<MW, 3><<<g, 256, 0, s>>>(disp, tS, tC, k.W, k.H, k.D, rs, rc, gate, k.gate_run);
 }
 
 // the column pass over nf frames: dst = the (2r+1)-row OR of the row results src
