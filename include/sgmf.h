@@ -197,7 +197,8 @@ sgmf_status sgmf_set_debug(sgmf_ctx *c, int enable);
  * sgmf_compute_batch (see SGMF_STAGE_*) into host memory host_dst of `bytes`
  * bytes; waits for the stream first.
  * Errors: SGMF_ERR_ARG for an unknown stage, a NULL destination, too few
- * bytes, or SGMF_STAGE_SUM without sgmf_set_debug(c, 1). */
+ * bytes, or SGMF_STAGE_SUM without sgmf_set_debug(c, 1); SGMF_ERR_OOM when a
+ * host buffer of a few MB cannot be had. */
 sgmf_status sgmf_debug_stage(sgmf_ctx *c, int stage, void *host_dst, size_t bytes);
 
 /* Number of kernel launches one sgmf_compute enqueues with the current

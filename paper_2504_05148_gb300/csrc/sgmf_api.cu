@@ -8,6 +8,7 @@
 #include <cstdlib>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <string>
 #include <vector>
@@ -735,6 +736,36 @@ extern "C" sgmf_status sgmf_set_debug(sgmf_ctx *c, int enable) {
   return SGMF_OK;
 }
 
+// n elements of src to the host through a buffer of bounded size: use(i0, values,
+// count) takes them block by block, blocks of whole units of `unit` elements
+template <typename T, typename F>
+static sgmf_status copy_blocks(sgmf_ctx *c, const T *src, size_t n, size_t unit, F &&use) {
+  constexpr size_t kBlock = size_t(1) << 20;
+  const size_t per = std::min(n, std::max<size_t>(1, kBlock / unit) * unit);
+  const std::unique_ptr<T[]> buf(new (std::nothrow) T[per]);
+  if (!buf) return fail(c, SGMF_ERR_OOM, "sgmf_debug_stage: host allocation failed");
+  for (size_t i = 0; i < n; i += per) {
+    const size_t m = std::min(per, n - i);
+    CUDA_TRY(c, cudaMemcpy(buf.get(), src + i, m * sizeof(T), cudaMemcpyDeviceToHost));
+    use(i, buf.get(), m);
+  }
+  return SGMF_OK;
+}
+
+// the first nd cells of n pixels' vectors of Dp cells, which lie in group-lane order
+template <typename T>
+static sgmf_status copy_vectors(sgmf_ctx *c, const T *src, size_t n, int nd, T *dst) {
+  const int Dp = c->k.Dp;
+  int cell[kMaxDisp];
+  for (int m = 0; m < Dp; ++m) cell[m] = lane_order_cell(Dp, sizeof(T) == 2, m);
+  return copy_blocks(c, src, n * Dp, Dp, [&](size_t i, const T *v, size_t count) {
+    T *o = dst + i / Dp * nd;
+    for (size_t j = 0; j < count; j += Dp, o += nd)
+      for (int m = 0; m < Dp; ++m)
+        if (cell[m] < nd) o[cell[m]] = v[j + m];
+  });
+}
+
 extern "C" sgmf_status sgmf_debug_stage(sgmf_ctx *c, int stage, void *dst, size_t bytes) {
   if (!c) return SGMF_ERR_ARG;
   if (!dst) return fail(c, SGMF_ERR_ARG, "sgmf_debug_stage: NULL destination");
@@ -782,30 +813,16 @@ extern "C" sgmf_status sgmf_debug_stage(sgmf_ctx *c, int stage, void *dst, size_
       if (k.census == SGMF_CENSUS_9X7) {
         CUDA_TRY(c, cudaMemcpy(dst, src, need, cudaMemcpyDeviceToHost));
       } else {
-        std::vector<uint32_t> tmp(n);
-        CUDA_TRY(c, cudaMemcpy(tmp.data(), src, n * 4, cudaMemcpyDeviceToHost));
         uint64_t *o = static_cast<uint64_t *>(dst);
-        for (size_t i = 0; i < n; ++i) o[i] = tmp[i];
+        return copy_blocks(c, static_cast<const uint32_t *>(src), n, 1, [&](size_t i, const uint32_t *v, size_t count) {
+          std::copy(v, v + count, o + i);
+        });
       }
       break;
     }
-    case SGMF_STAGE_COST:
-    case SGMF_STAGE_SUM: {
-      const bool u16 = stage == SGMF_STAGE_SUM;
-      const void *src = u16 ? static_cast<const void *>(c->b.dbg_sum) : c->b.cost;
-      // Dp cells a pixel in group-lane order (banded: Dp = band, cell j = disparity lo_p + j)
-      const int nd = k.band ? k.band : k.D;
-      const size_t es = u16 ? 2 : 1;
-      std::vector<uint8_t> tmp(n * k.Dp * es);
-      CUDA_TRY(c, cudaMemcpy(tmp.data(), src, tmp.size(), cudaMemcpyDeviceToHost));
-      std::vector<int> cell(k.Dp);
-      for (int m = 0; m < k.Dp; ++m) cell[m] = lane_order_cell(k.Dp, u16, m);
-      for (size_t p = 0; p < n; ++p)
-        for (int m = 0; m < k.Dp; ++m)
-          if (cell[m] < nd)
-            memcpy(static_cast<uint8_t *>(dst) + (p * nd + cell[m]) * es, &tmp[(p * k.Dp + m) * es], es);
-      break;
-    }
+    // (banded: Dp = band, cell j = disparity lo_p + j)
+    case SGMF_STAGE_COST: return copy_vectors(c, c->b.cost, n, k.band ? k.band : k.D, static_cast<uint8_t *>(dst));
+    case SGMF_STAGE_SUM: return copy_vectors(c, c->b.dbg_sum, n, k.band ? k.band : k.D, static_cast<uint16_t *>(dst));
   }
   return SGMF_OK;
 }
