@@ -59,18 +59,30 @@ TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic_kitti_1242x375_d128.txt")
 # ops:   scalar integer operations of the method (Eq. 2: 2 adds of P1, 3 mins,
 #        1 add of C, 1 subtraction of m and 1 min toward the next m = 8 per cell
 #        and direction; the path sum 1 add per cell and direction; WTA 2 mins per cell).
-def algorithmic(name: str, V: int, N: int, num_paths: int = 8, sweep: bool = False):
+# form: sgmf_agg_form's fields, with row_walks as the fraction of the frames whose rows
+#       are line walks; None: the default line walks with byte costs.
+def algorithmic(name: str, V: int, N: int, num_paths: int = 8, form: dict | None = None):
+    f = form or {"sweep": 0, "row_walks": 1.0, "half_rows": 0, "half_lines": 0, "cost_bytes": 1}
+    walks = f["row_walks"]                                   # part of the frames
+    lines = 0 if f["sweep"] else num_paths - 2               # vertical and diagonal directions walked
+    rows_kept, lines_kept = (0.5 if f["half_rows"] else 1.0), (0.5 if f["half_lines"] else 1.0)
+    # bytes of the vectors that the walks write and the winner kernel reads, per cell
+    vectors = f["cost_bytes"] * (2 * rows_kept + lines * lines_kept)
     if name == "agg_lines":
-        # the cost volume read once, one byte vector per direction written
-        return {"bytes": V * 1 + num_paths * V, "ops": 8 * num_paths * V}
+        # the cost volume read once, the stored vectors of each walked direction written
+        return {"bytes": walks * V * (1 + vectors), "ops": walks * V * 8 * (2 + lines)}
     if name == "agg_sweep":
         # the cost volume read once, two u16 sums of three directions written
         return {"bytes": V * 1 + 2 * 2 * V, "ops": 8 * 6 * V + 4 * V}
     if name == "agg_rows_wta":
-        if not sweep:                    # every direction's byte vectors read, summed, WTA
-            return {"bytes": num_paths * V + 4 * N, "ops": num_paths * V + 2 * V}
-        # the row walks, and two u16 sums of three directions read
-        return {"bytes": V * 1 + 2 * 2 * V + 4 * N, "ops": 8 * 2 * V + 4 * V + 2 * V}
+        sums = 2 * 2 if f["sweep"] else 0                    # two u16 sums of three directions read
+        # the winner kernel: the stored vectors read, the steps of those left out (on the costs), the sum, WTA
+        left_out = 2 * (1 - rows_kept) + lines * (1 - lines_kept)
+        wta = {"bytes": V * (vectors + sums + (1 if left_out else 0)) + 4 * N,
+               "ops": V * (8 * left_out + 2 + lines + sums / 2 + 2)}
+        # the row kernel: both row directions walked, the sums read, the sum, WTA
+        rows = {"bytes": V * (1 + sums) + 4 * N, "ops": V * (8 * 2 + 4 + 2)}
+        return {k: walks * wta[k] + (1 - walks) * rows[k] for k in wta}
     if name == "cost":
         return {"bytes": V + 4 * N * 2 + 2 * N, "ops": 4 * V}
     return None
@@ -959,7 +971,10 @@ def main():
     tot = {k: sum(v) for k, v in ktimes.items()}
     dom = max(tot, key=tot.get)
     V, N = W * H * D * B, W * H * B          # every launch covers the B frames of a step
-    alg = algorithmic(dom, V, N, sweep=tuning is not None and len(tuning) > 2 and tuning[2] == 1)
+    form = sgmf.sgmf_get_agg_form(ctx.handle, B)
+    form = {k: getattr(form, k) for k, _ in form._fields_}
+    form["row_walks"] /= B
+    alg = algorithmic(dom, V, N, form=form)
     sm_mhz = (clk or {}).get("sm_mhz") or peaks["sm_max_mhz"]
     alu_peak = 152 * 64 * 2 * sm_mhz * 1e6       # u16x2 lanes of the ALU pipe, per second
     roof = None

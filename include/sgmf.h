@@ -205,6 +205,18 @@ sgmf_status sgmf_debug_stage(sgmf_ctx *c, int stage, void *host_dst, size_t byte
  * parameters (for launch accounting). */
 int sgmf_launches_per_compute(const sgmf_ctx *c);
 
+/* What the aggregation of a call of n frames (1 <= n <= the batch capacity)
+ * moves and computes, with the context's parameters and tuning: for work counts. */
+typedef struct {
+    int32_t sweep;       /* 1: the vertical and diagonal directions are cluster sweeps */
+    int32_t row_walks;   /* frames whose rows are line walks (n without the sweep), the
+                            winner kernel behind them; the other frames' rows are the row kernel's */
+    int32_t half_rows;   /* 1: of the rows' walks every second column's vectors are stored */
+    int32_t half_lines;  /* 1: of the other directions' walks every second row's */
+    int32_t cost_bytes;  /* bytes of a stored path cost: 1 or 2 */
+} sgmf_agg_form;
+sgmf_status sgmf_get_agg_form(const sgmf_ctx *c, int n, sgmf_agg_form *form);
+
 /* Record CUDA events around every kernel of the following sgmf_compute
  * calls (enable = 1) or stop (0). */
 sgmf_status sgmf_set_profiling(sgmf_ctx *c, int enable);

@@ -596,6 +596,21 @@ static int half_vectors(const sgmf_ctx *c, int n) {
   return !k.band && (k.Dp == 128 || k.Dp == 192) && cells >= (k.num_paths == 8 ? 100000000u : 200000000u);
 }
 
+extern "C" sgmf_status sgmf_get_agg_form(const sgmf_ctx *c, int n, sgmf_agg_form *form) {
+  if (!c || !form || n < 1 || n > c->nb) return SGMF_ERR_ARG;
+  *form = {};
+  form->sweep = use_sweep(c);
+  form->cost_bytes = c->spill8 ? 1 : 2;
+  form->half_lines = !form->sweep && half_vectors(c, n);
+  form->half_rows = form->half_lines || !c->spill8;
+  const int part = form->sweep ? sweep_part(c, n) : 0, m = part > 0 ? part : n;
+  for (int f0 = 0; f0 < n; f0 += m) {
+    const int nf = std::min(m, n - f0);
+    if (!form->sweep || rows_as_lines(c, nf)) form->row_walks += nf;
+  }
+  return SGMF_OK;
+}
+
 // Aggregation, winners and check of the n frames whose cost volume is made.
 // A sweep batch goes through in parts of m frames: part i's sweep on the
 // context's stream, then the rest of it on the side stream while part i + 1 is

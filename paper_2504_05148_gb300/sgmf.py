@@ -31,7 +31,7 @@ EXPORTS = (
     "sgmf_default_params", "sgmf_create", "sgmf_create_batched", "sgmf_batch_capacity", "sgmf_set_params",
     "sgmf_get_params", "sgmf_set_stream", "sgmf_compute", "sgmf_compute_batch", "sgmf_compute_host",
     "sgmf_compute_host_batch", "sgmf_sync", "sgmf_destroy", "sgmf_last_error",
-    "sgmf_status_string", "sgmf_set_debug", "sgmf_debug_stage", "sgmf_launches_per_compute",
+    "sgmf_status_string", "sgmf_set_debug", "sgmf_debug_stage", "sgmf_launches_per_compute", "sgmf_get_agg_form",
     "sgmf_set_profiling", "sgmf_kernel_times", "sgmf_device_bytes", "sgmf_check_static",
     "sgmf_set_wait_limit", "sgmf_debug_fail_alloc", "sgmf_measure_rates",
     "sgmf_set_tuning", "sgmf_get_tuning", "sgmf_autotune",
@@ -67,6 +67,10 @@ class sgmf_rates(ctypes.Structure):
 class sgmf_tuning(ctypes.Structure):
     _fields_ = [("line_warps", ctypes.c_int32), ("cost_px", ctypes.c_int32), ("sweep", ctypes.c_int32),
                 ("parts", ctypes.c_int32)]
+
+
+class sgmf_agg_form(ctypes.Structure):
+    _fields_ = [(k, ctypes.c_int32) for k in ("sweep", "row_walks", "half_rows", "half_lines", "cost_bytes")]
 
 
 class sgmf_server_counters(ctypes.Structure):
@@ -151,6 +155,7 @@ def lib(path: str | None = None):
         "sgmf_set_debug": (i, [P, i]),
         "sgmf_debug_stage": (i, [P, i, P, sz]),
         "sgmf_launches_per_compute": (i, [P]),
+        "sgmf_get_agg_form": (i, [P, i, ctypes.POINTER(sgmf_agg_form)]),
         "sgmf_set_profiling": (i, [P, i]),
         "sgmf_kernel_times": (i, [P, ctypes.POINTER(ctypes.c_char_p), ctypes.POINTER(ctypes.c_float),
                                   ctypes.POINTER(ctypes.c_int)]),
@@ -306,6 +311,12 @@ def sgmf_debug_stage(ctx: int, stage: int, host_ptr: int, nbytes: int) -> None:
 
 def sgmf_launches_per_compute(ctx: int) -> int:
     return lib().sgmf_launches_per_compute(ctx)
+
+
+def sgmf_get_agg_form(ctx: int, n: int) -> sgmf_agg_form:
+    form = sgmf_agg_form()
+    _check(lib().sgmf_get_agg_form(ctx, n, ctypes.byref(form)), ctx)
+    return form
 
 
 def sgmf_set_profiling(ctx: int, enable: bool) -> None:
