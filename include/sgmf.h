@@ -421,18 +421,20 @@ typedef struct {
                              segments of up to 1024 pixels) */
     int32_t sweep;        /* 1: the six vertical and diagonal directions run as two
                              row-synchronous sweeps of a thread-block cluster per
-                             frame (one launch) instead of their line walks
-                             (line_warps is then unused).  0 (default) or 1; 1 needs
-                             a row of at most 16 CTAs x 128 pixels (Dp <= 128) or
-                             16 x 80 pixels (Dp > 128; banded: 16 x 160) and
+                             frame (one launch) instead of their line walks.  The
+                             rows behind it are the row kernel's or, in calls of
+                             few rows a SM, line walks (which line_warps shapes).
+                             0 (default) or 1; 1 needs a row of at most 16 CTAs x
+                             128 pixels (Dp <= 128) or 16 x 80 pixels (Dp > 128) and
                              a device that can place such a cluster (the context
                              picks the cluster size that keeps the most CTAs
                              resident), and is refused otherwise; it takes effect
-                             with 8 paths on a plain context (a banded one walks
-                             lines, which is faster there). */
+                             with 8 paths on a plain context.  A banded context
+                             accepts 1 for rows of up to 2560 pixels and walks
+                             lines all the same, which is faster there. */
     int32_t parts;        /* with the sweep: 1 (default) runs a batch in parts of one
-                             sweep wave, each part's row kernel on a second stream
-                             beside the next part's sweep; 0 runs the whole batch
+                             sweep wave, what follows a part's sweep on a second
+                             stream beside the next part's; 0 runs the whole batch
                              through each kernel in one launch.  0 or 1. */
 } sgmf_tuning;
 
@@ -442,7 +444,8 @@ sgmf_status sgmf_get_tuning(const sgmf_ctx *c, sgmf_tuning *t);
 
 /* Autotuner.  Runs sgmf_compute_batch(c, n, left, right, lidar, out) on the
  * caller's DEVICE frames once per candidate (the 4 x 3 line-kernel tunings,
- * and the sweep with each of the 3 cost shapes where it fits) as a
+ * and the sweep with each of the 3 cost shapes where it fits, with the
+ * line_warps that the context has) as a
  * warm-up, then `reps` timed runs, each after overwriting up to 256 MiB of
  * the context's scratch so that it starts with a cold L2 (CUDA events on the
  * context's stream, 1 <= reps <= 100); keeps the candidate with the smallest median time in

@@ -292,8 +292,8 @@ class LearnedSGM:
         # one banded context per width (gate value = its index), the plain one last
         self.ctxs = [S.Context(W, H, D, params, band=b, max_batch=max_batch) for b in self.bands]
         self.banded = self.ctxs[0]          # runs the front half that feeds the network
-        # the cluster sweep for the banded walks where it fits; it needs several
-        # frames per call to fill the GPU (one cluster per frame and direction)
+        # a launch tuning that banded contexts of up to 2560 columns accept and that
+        # changes nothing: their directions are line walks either way
         if sweep if sweep is not None else max_batch >= 4:
             for c in self.ctxs:
                 try:

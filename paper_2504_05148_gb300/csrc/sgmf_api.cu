@@ -246,6 +246,9 @@ static cudaError_t side_stream(cudaStream_t *s) {
   return cudaStreamCreateWithPriority(s, cudaStreamNonBlocking, kSidePriority ? greatest : least);
 }
 
+// rows up to which a banded context accepts the sweep tuning: what its own sweep
+// took while there was one.  The tuning has no effect there (use_sweep); the
+// calls that accept and refuse it stay as they were
 constexpr int kMaxBandSweepRow = 2560;
 
 static sgmf_status create_ctx(int width, int height, int max_disp, int max_batch, int band, sgmf_ctx **out) {

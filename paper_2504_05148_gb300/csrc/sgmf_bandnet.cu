@@ -158,7 +158,6 @@ __device__ __forceinline__ uint32_t f2bf2(float lo, float hi) {
   const __nv_bfloat162 b = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t *>(&b);
 }
-__device__ __forceinline__ float bf2f(uint16_t u) { return __uint_as_float((uint32_t)u << 16); }
 
 // ---- weights -> B images ------------------------------------------------------------
 // w: bf16 [co][ky][kx][ci].  fwd image: row co, k = tap * 32 + ci.  dgrad

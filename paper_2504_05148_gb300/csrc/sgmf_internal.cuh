@@ -32,7 +32,6 @@ constexpr int kMaxDim = 8192;
 // banded mode: the band start is constant on kBandTile x kBandTile pixel tiles
 constexpr int kBandTileLog = 3, kBandTile = 1 << kBandTileLog;
 constexpr uint32_t kInf = 0x4000u;          // u16 lane value above every real path cost
-constexpr uint32_t kInf2 = kInf | (kInf << 16);
 
 enum ErrorCode : int { kErrNone = 0, kErrTimeout = 6 };
 
@@ -270,12 +269,6 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
       : "memory");
 }
 
-// order this thread's earlier generic-proxy global writes before later
-// async-proxy (bulk copy) reads of the same data
-__device__ __forceinline__ void fence_proxy_async_global() {
-  asm volatile("fence.proxy.async.global;" ::: "memory");
-}
-
 // order this thread's earlier shared-memory writes before later async-proxy
 // (bulk copy) reads of them
 __device__ __forceinline__ void fence_proxy_async_shared() {
@@ -321,8 +314,6 @@ inline cudaError_t once_per_device(bool (&done)[64], F &&setup) {
 cudaError_t sm_count(int *out);
 
 // ---- kernel launchers (implemented in the .cu files) -----------------------
-struct TmaMaps;   // opaque holder of the two image tensor maps (sgmf_front.cu)
-
 // Every launcher covers frames [0, nf) of the context's buffers.
 // C-bar of Eq. 4 by q class (0: d = prior, 1: |d - prior| = 1, 2: farther)
 // and Hamming distance H; class 3 (no prior) is the identity, C-bar = H:

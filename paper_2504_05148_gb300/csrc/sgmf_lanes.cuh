@@ -63,18 +63,16 @@ struct Raw8 {
   uint32_t v[CPL / 4];
 };
 
-template <int CPL, bool NC>
+template <int CPL>
 __device__ __forceinline__ void load_raw8(const uint8_t *p, Raw8<CPL> &r) {
   using V = Vec8<CPL>;
 #pragma unroll
   for (int q = 0; q < V::N; ++q) {
     if constexpr (V::CH == 16) {
-      const uint4 *s = reinterpret_cast<const uint4 *>(p + q * V::kNext);
-      const uint4 t = NC ? __ldg(s) : *s;
+      const uint4 t = *reinterpret_cast<const uint4 *>(p + q * V::kNext);
       r.v[4 * q] = t.x, r.v[4 * q + 1] = t.y, r.v[4 * q + 2] = t.z, r.v[4 * q + 3] = t.w;
     } else {
-      const uint2 *s = reinterpret_cast<const uint2 *>(p + q * V::kNext);
-      const uint2 t = NC ? __ldg(s) : *s;
+      const uint2 t = *reinterpret_cast<const uint2 *>(p + q * V::kNext);
       r.v[2 * q] = t.x, r.v[2 * q + 1] = t.y;
     }
   }
@@ -94,7 +92,7 @@ __device__ __forceinline__ void expand8(const Raw8<CPL> &r, const uint32_t (&z)[
 template <int CPL>
 __device__ __forceinline__ void load_u8(const uint8_t *p, const uint32_t (&z)[CPL / 4], uint32_t (&w)[CPL / 2]) {
   Raw8<CPL> r;
-  load_raw8<CPL, false>(p, r);
+  load_raw8<CPL>(p, r);
   expand8<CPL>(r, z, w);
 }
 
@@ -115,16 +113,6 @@ __device__ __forceinline__ void store_u8(uint8_t *p, const uint32_t (&w)[CPL / 2
 }
 
 template <int CPL>
-__device__ __forceinline__ void load_u16(const uint8_t *p, uint32_t (&w)[CPL / 2]) {
-  using V = Vec16<CPL>;
-#pragma unroll
-  for (int q = 0; q < V::N; ++q) {
-    const uint4 t = *reinterpret_cast<const uint4 *>(p + q * V::kNext);
-    w[4 * q] = t.x, w[4 * q + 1] = t.y, w[4 * q + 2] = t.z, w[4 * q + 3] = t.w;
-  }
-}
-
-template <int CPL>
 __device__ __forceinline__ void store_u16(uint8_t *p, const uint32_t (&w)[CPL / 2]) {
   using V = Vec16<CPL>;
 #pragma unroll
@@ -135,20 +123,12 @@ __device__ __forceinline__ void store_u16(uint8_t *p, const uint32_t (&w)[CPL / 
 // a vector in the width its path costs need: bytes (S8) or u16
 template <int CPL, bool S8>
 struct VecW {
-  static constexpr int kLane = S8 ? Vec8<CPL>::kLane : Vec16<CPL>::kLane, SB = S8 ? 1 : 2;
+  static constexpr int kLane = S8 ? Vec8<CPL>::kLane : Vec16<CPL>::kLane;
   static __device__ __forceinline__ void put(uint8_t *p, const uint32_t (&w)[CPL / 2]) {
     if constexpr (S8)
       store_u8<CPL>(p, w);
     else
       store_u16<CPL>(p, w);
-  }
-  static __device__ __forceinline__ void get(const uint8_t *p, uint32_t (&w)[CPL / 2]) {
-    if constexpr (S8) {
-      const uint32_t z[CPL / 4] = {};
-      load_u8<CPL>(p, z, w);
-    } else {
-      load_u16<CPL>(p, w);
-    }
   }
 };
 
@@ -246,7 +226,7 @@ __device__ __forceinline__ uint32_t mad_u32(uint32_t a, uint32_t b, uint32_t c) 
 
 // The group's outer neighbours, as bits ORed into the first / last lane's words:
 // 0xffff in the missing neighbour's half (L(-1), L(Dp) only enter a min).  On the
-// bands the neighbour's half is cleared first (keep) and may hold the previous
+// bands the neighbour's half is cleared first (step) and may hold the previous
 // pixel's cell just outside the current band (band_shift).
 struct Edges {
   uint32_t lo, hi;

@@ -27,13 +27,13 @@
 namespace sgmf {
 namespace oct {
 
-constexpr int kMaxVec = 2;      // u16 vectors (the sweep's sums) read per pixel beside cost and spill
+constexpr int kSums = 2;        // u16 vectors (the sweep's sums) read per pixel beside cost and spill
 
 struct RowArgs {
   KParams k;
   const uint8_t *cost;
-  const uint8_t *vec[kMaxVec];  // frame 0's vertical / diagonal vectors, 2 Dp bytes per pixel
-  size_t vec_frame[kMaxVec];    // bytes from one frame to the next
+  const uint8_t *vec[kSums];  // frame 0's vertical / diagonal vectors, 2 Dp bytes per pixel
+  size_t vec_frame[kSums];    // bytes from one frame to the next
   uint8_t *spill;               // frame 0's row spill region
   size_t spill_frame;
   int16_t *dstar, *dprime;
@@ -43,13 +43,13 @@ struct RowArgs {
   const int *gate;              // per-frame gate words of the launch's frames, or null
 };
 
-// NV: u16 vectors added.  A slot holds, for the 32 lanes of a warp, the
-// pieces of one step: cost bytes, spill, vectors.
-template <int CPL, bool S8, int NV>
+// A slot holds, for the 32 lanes of a warp, the pieces of one step: cost bytes,
+// spill, the sums.
+template <int CPL, bool S8>
 struct RowCfg {
   static constexpr int Dp = kGL * CPL, SB = S8 ? 1 : 2;
   static constexpr int k8 = 32 * CPL, k16 = 2 * k8;              // bytes of a byte / u16 vector of the four rows
-  static constexpr int oSpill = k8, oVec = oSpill + (S8 ? k8 : k16), kSlot = oVec + NV * k16;
+  static constexpr int oSpill = k8, oVec = oSpill + (S8 ? k8 : k16), kSlot = oVec + kSums * k16;
   // slots: up to 8 steps (at least 2) in about 32 KB a warp
   static constexpr int R = 8 * kSlot <= 32768 ? 8 : (4 * kSlot <= 32768 ? 4 : 2);
   static constexpr int U = R < 4 ? R : 4;                        // steps unrolled
@@ -78,13 +78,13 @@ struct RowLane {
   uint8_t *spill;               // the lane's first chunk of the row's spill
   uint8_t *dbg;                 // and of its S, or null
   int16_t *dstar, *dprime, *dsub;
-  const uint8_t *cost, *vec[kMaxVec];   // the lane's first chunk of the row's pixel 0
+  const uint8_t *cost, *vec[kSums];   // the lane's first chunk of the row's pixel 0
   uint32_t *merge;              // the row's merge words; word i: right pixel xm - D + 1 + i
 };
 
-template <int CPL, bool S8, int NV, bool FWD, bool SECOND>
+template <int CPL, bool S8, bool FWD, bool SECOND>
 __device__ __forceinline__ void row_step(RowWalk<CPL> &w, const RowLane<CPL> &g, const uint8_t *slot, int x) {
-  using CF = RowCfg<CPL, S8, NV>;
+  using CF = RowCfg<CPL, S8>;
   constexpr int NW = CPL / 2, Dp = CF::Dp;
   const uint32_t z0[CPL / 4] = {};
   uint32_t C[NW];
@@ -102,7 +102,7 @@ __device__ __forceinline__ void row_step(RowWalk<CPL> &w, const RowLane<CPL> &g,
 #pragma unroll
     for (int i = 0; i < NW; ++i) Sm[i] += w.L[i];
 #pragma unroll
-    for (int j = 0; j < NV; ++j) {
+    for (int j = 0; j < kSums; ++j) {
       const uint8_t *v = slot + CF::oVec + j * CF::k16;
       uint32_t T[NW];
       slot16<CPL>(v, g.lane, T);
@@ -176,16 +176,16 @@ __device__ __forceinline__ void row_step(RowWalk<CPL> &w, const RowLane<CPL> &g,
 
 // One half of a warp's walk over n pixels from x0 on: SECOND the pixels the
 // other warp reached first.
-template <int CPL, bool S8, int NV, bool FWD, bool SECOND>
+template <int CPL, bool S8, bool FWD, bool SECOND>
 __device__ __forceinline__ void row_half(RowWalk<CPL> &w, const RowLane<CPL> &g, uint8_t *ring, int x0, int n) {
-  using CF = RowCfg<CPL, S8, NV>;
+  using CF = RowCfg<CPL, S8>;
   constexpr int R = CF::R, U = CF::U, Dp = CF::Dp, kMove = FWD ? 1 : -1;
   const uint32_t ring_s = smem_u32(ring);
   // sources of the next step to copy
   const uint8_t *pc = g.cost + (ptrdiff_t)x0 * Dp, *ps = g.spill + (ptrdiff_t)x0 * Dp * CF::SB;
-  const uint8_t *pv[NV];
+  const uint8_t *pv[kSums];
 #pragma unroll
-  for (int j = 0; j < NV; ++j) pv[j] = g.vec[j] + (ptrdiff_t)x0 * 2 * Dp;
+  for (int j = 0; j < kSums; ++j) pv[j] = g.vec[j] + (ptrdiff_t)x0 * 2 * Dp;
   auto copy = [&](uint32_t slot) {
     copy8<CPL>(slot, g.lane, pc);
     pc += kMove * Dp;
@@ -196,7 +196,7 @@ __device__ __forceinline__ void row_half(RowWalk<CPL> &w, const RowLane<CPL> &g,
         copy16<CPL>(slot + CF::oSpill, g.lane, ps);
       ps += kMove * Dp * CF::SB;
 #pragma unroll
-      for (int j = 0; j < NV; ++j) {
+      for (int j = 0; j < kSums; ++j) {
         copy16<CPL>(slot + CF::oVec + j * CF::k16, g.lane, pv[j]);
         pv[j] += kMove * 2 * Dp;
       }
@@ -212,7 +212,7 @@ __device__ __forceinline__ void row_half(RowWalk<CPL> &w, const RowLane<CPL> &g,
     for (int u = 0; u < U; ++u) {
       if (t + u >= n) break;
       cp_wait<R - 1>();
-      row_step<CPL, S8, NV, FWD, SECOND>(w, g, ring + base + u * CF::kSlot, x0 + kMove * (t + u));
+      row_step<CPL, S8, FWD, SECOND>(w, g, ring + base + u * CF::kSlot, x0 + kMove * (t + u));
       if (t + u + R < n) copy(ring_s + base + u * CF::kSlot);
       cp_commit();
     }
@@ -222,7 +222,7 @@ __device__ __forceinline__ void row_half(RowWalk<CPL> &w, const RowLane<CPL> &g,
 }
 
 // One warp's walk of its four rows.
-template <int CPL, bool S8, int NV, bool FWD>
+template <int CPL, bool S8, bool FWD>
 __device__ __forceinline__ void row_walk(const RowLane<CPL> &g, uint8_t *ring) {
   RowWalk<CPL> w;
 #pragma unroll
@@ -230,9 +230,9 @@ __device__ __forceinline__ void row_walk(const RowLane<CPL> &g, uint8_t *ring) {
   w.mm = 0u;
 #pragma unroll
   for (int j = 0; j < CPL; ++j) w.acc[j] = 0xffffffffu;
-  row_half<CPL, S8, NV, FWD, false>(w, g, ring, FWD ? 0 : g.W - 1, FWD ? g.xm : g.W - g.xm);
+  row_half<CPL, S8, FWD, false>(w, g, ring, FWD ? 0 : g.W - 1, FWD ? g.xm : g.W - g.xm);
   __syncthreads();                               // both first halves are stored
-  row_half<CPL, S8, NV, FWD, true>(w, g, ring, FWD ? g.xm : g.xm - 1, FWD ? g.W - g.xm : g.xm);
+  row_half<CPL, S8, FWD, true>(w, g, ring, FWD ? g.xm : g.xm - 1, FWD ? g.W - g.xm : g.xm);
   if (FWD && g.act) {
     // right pixels x' = W-1-d whose diagonal leaves the image: the slots left
 #pragma unroll
@@ -248,9 +248,9 @@ __device__ __forceinline__ void row_walk(const RowLane<CPL> &g, uint8_t *ring) {
   }
 }
 
-template <int CPL, bool S8, int NV>
+template <int CPL, bool S8>
 __global__ void __launch_bounds__(64) k_rows(const __grid_constant__ RowArgs a) {
-  using CF = RowCfg<CPL, S8, NV>;
+  using CF = RowCfg<CPL, S8>;
   constexpr int Dp = CF::Dp, NW = CPL / 2;
   extern __shared__ __align__(128) uint8_t smem[];
   const int f = blockIdx.y;
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(64) k_rows(const __grid_constant__ RowArgs a) 
   g.cost = a.cost + f * fcells + g.row * Dp + lig * Vec8<CPL>::kLane;
   g.spill = a.spill + f * a.spill_frame + g.row * Dp * CF::SB + lig * VecW<CPL, S8>::kLane;
 #pragma unroll
-  for (int j = 0; j < NV; ++j)
+  for (int j = 0; j < kSums; ++j)
     g.vec[j] = a.vec[j] + f * a.vec_frame[j] + g.row * 2 * Dp + lig * Vec16<CPL>::kLane;
   g.dbg = (f == 0 && a.dbg_sum != nullptr)
               ? reinterpret_cast<uint8_t *>(a.dbg_sum) + g.row * Dp * 2 + lig * Vec16<CPL>::kLane
@@ -293,9 +293,9 @@ __global__ void __launch_bounds__(64) k_rows(const __grid_constant__ RowArgs a) 
   for (int i = threadIdx.x; i < kGW * Dp; i += blockDim.x) merge[i] = 0xffffffffu;
   __syncthreads();
   if (warp == 0)
-    row_walk<CPL, S8, NV, true>(g, smem);
+    row_walk<CPL, S8, true>(g, smem);
   else
-    row_walk<CPL, S8, NV, false>(g, smem + CF::R * CF::kSlot);
+    row_walk<CPL, S8, false>(g, smem + CF::R * CF::kSlot);
   __syncthreads();
   // right pixels whose diagonal crosses the middle: both warps contributed
   for (int r = warp; r < kGW && y0 + r < a.k.H; r += 2)
@@ -306,13 +306,13 @@ __global__ void __launch_bounds__(64) k_rows(const __grid_constant__ RowArgs a) 
     }
 }
 
-template <int CPL, bool S8, int NV>
+template <int CPL, bool S8>
 static cudaError_t launch_rows_v(const RowArgs &a, int nf, cudaStream_t s) {
-  using CF = RowCfg<CPL, S8, NV>;
+  using CF = RowCfg<CPL, S8>;
   static bool done[64] = {};
-  cudaError_t e = smem_optin(k_rows<CPL, S8, NV>, CF::kSmem, done);
+  cudaError_t e = smem_optin(k_rows<CPL, S8>, CF::kSmem, done);
   if (e != cudaSuccess) return e;
-  k_rows<CPL, S8, NV><<<dim3((a.k.H + kGW - 1) / kGW, nf), 64, CF::kSmem, s>>>(a);
+  k_rows<CPL, S8><<<dim3((a.k.H + kGW - 1) / kGW, nf), 64, CF::kSmem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -330,11 +330,11 @@ cudaError_t launch_rows_t(const KParams &k, const Buffers &b, int nf, cudaStream
   a.dbg_sum = b.dbg_sum;
   a.sc = step_consts(k);
   a.gate = b.gate;
-  for (int i = 0; i < 2; ++i) {
+  for (int i = 0; i < kSums; ++i) {
     a.vec[i] = reinterpret_cast<const uint8_t *>(b.part[i]);
     a.vec_frame[i] = 2 * cells;
   }
-  return launch_rows_v<CPL, S8, 2>(a, nf, s);
+  return launch_rows_v<CPL, S8>(a, nf, s);
 }
 
 }  // namespace oct
