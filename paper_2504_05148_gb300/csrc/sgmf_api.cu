@@ -32,8 +32,8 @@ struct sgmf_ctx {
   bool sweep_ok = false;       // the row-synchronous sweep can run this shape on this device (8 paths)
   int sweep_slots = 0;         // sweep clusters the device holds at once
   size_t spill_bytes = 0;
-  // with the sweep, a batch goes through in parts: part i's row kernel and
-  // check run on this second stream while part i + 1 is in the sweep
+  // with the sweep, a batch goes through in parts: what follows part i's sweep
+  // (finish) runs on this second stream while part i + 1 is in the sweep
   static constexpr int kMaxParts = 8;
   cudaStream_t side = nullptr;
   cudaEvent_t ev_part[kMaxParts] = {};
@@ -426,7 +426,7 @@ static bool need_boxc(const KParams &k) { return k.consistency == SGMF_CHECK_STE
 static bool use_sweep(const sgmf_ctx *c) { return c->k.sweep && c->k.num_paths == 8 && c->sweep_ok && !c->k.band; }
 
 // Frames per part when a sweep batch of n frames goes through in parts (0:
-// one part).  A part's row kernel and check run on the side stream beside
+// one part).  What follows a part's sweep runs on the side stream beside
 // the next part's sweep, filling the SMs (and the register room) the sweep
 // clusters leave.  Every part but the last is one wave of sweep clusters
 // (2 m cluster jobs, the resident count or its smallest even multiple), so

@@ -1,5 +1,5 @@
 // sgmf_lanes.cuh -- the lane layout and the recursion step (Eq. 2) of the
-// full-range aggregation kernels.
+// aggregation kernels, over the full range and on the bands.
 //
 // A group of 8 lanes holds the Dp disparities of one path-cost vector; lane j
 // holds cells [j CPL, (j + 1) CPL), CPL = Dp / 8, as NW = CPL / 2 u16x2 words.
