@@ -486,8 +486,10 @@ sgmf_status sgmf_multi_class_info(const sgmf_multi *m, int cls, sgmf_shape *shap
                                   sgmf_tuning *t);
 
 /* sgmf_autotune for every class on its resident frames (`reps` timed runs
- * per candidate); drops a captured graph so that the next launch recaptures
- * with the chosen tunings.  Synchronous. */
+ * per candidate), then the sweep or the line walks for each class where both
+ * fit, by the time of the whole batch (at least 5 timed runs per candidate);
+ * drops a captured graph so that the next launch recaptures with the chosen
+ * tunings.  Synchronous. */
 sgmf_status sgmf_multi_autotune(sgmf_multi *m, int reps);
 
 /* Runs the whole batch on `stream` (NULL = the batch's own stream) as one

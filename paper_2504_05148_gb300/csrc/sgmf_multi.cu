@@ -9,6 +9,7 @@
 // batched context expects), so the captured pointers never change.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdarg>
 #include <cstdio>
 #include <map>
@@ -177,17 +178,6 @@ extern "C" sgmf_status sgmf_multi_class_info(const sgmf_multi *m, int cls, sgmf_
   return SGMF_OK;
 }
 
-extern "C" sgmf_status sgmf_multi_autotune(sgmf_multi *m, int reps) {
-  if (!m) return mfail(SGMF_ERR_ARG, "sgmf_multi_autotune: NULL batch");
-  if (m->last) cudaStreamSynchronize(m->last);
-  drop_graph(m);
-  for (MultiClass &c : m->cls) {
-    sgmf_status st = sgmf_autotune(c.ctx, c.nf, c.left, c.right, c.lidar, c.out, reps, nullptr, nullptr);
-    if (st != SGMF_OK) return mfail(st, "sgmf_multi_autotune: %s", sgmf_last_error(c.ctx));
-  }
-  return SGMF_OK;
-}
-
 // every class once on its own stream, outside any capture: first-use kernel
 // attributes are set here, not inside the capture
 static sgmf_status run_classes(sgmf_multi *m) {
@@ -234,6 +224,75 @@ static sgmf_status capture(sgmf_multi *m) {
     return mfail(SGMF_ERR_CUDA, "sgmf_multi_launch: instantiate: %s", cudaGetErrorString(e));
   }
   return SGMF_OK;
+}
+
+// median time of the whole batch as a graph with the classes' present tunings
+static sgmf_status time_batch(sgmf_multi *m, int reps, float *ms) {
+  drop_graph(m);
+  sgmf_status st = run_classes(m);
+  if (st == SGMF_OK) st = capture(m);
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  cudaError_t e = cudaSuccess;
+  auto cuda = [&](cudaError_t r) {
+    if (e == cudaSuccess) e = r;
+  };
+  std::vector<float> t;
+  if (st == SGMF_OK) {
+    cuda(cudaEventCreate(&e0));
+    cuda(cudaEventCreate(&e1));
+    const int runs = std::max(reps, 5);                     // (overlapping classes vary from run to run)
+    for (int r = 0; r <= runs && e == cudaSuccess; ++r) {   // the first is a warm-up
+      float v = 0.0f;
+      cuda(cudaEventRecord(e0, m->origin));
+      cuda(cudaGraphLaunch(m->exec, m->origin));
+      cuda(cudaEventRecord(e1, m->origin));
+      cuda(cudaEventSynchronize(e1));
+      cuda(cudaEventElapsedTime(&v, e0, e1));
+      if (r > 0) t.push_back(v);
+    }
+  }
+  if (e0) cudaEventDestroy(e0);
+  if (e1) cudaEventDestroy(e1);
+  drop_graph(m);
+  if (st != SGMF_OK) return st;
+  if (e != cudaSuccess) return mfail(SGMF_ERR_CUDA, "sgmf_multi_autotune: %s", cudaGetErrorString(e));
+  std::sort(t.begin(), t.end());
+  *ms = t[t.size() / 2];
+  return SGMF_OK;
+}
+
+// Each class's best launch shape alone, then the sweep or the line walks for
+// each class by the time of the whole batch: a class alone prefers the walks where
+// they are DRAM-bound, beside other classes that are DRAM-bound too the sweep,
+// which moves fewer bytes (12 pairs each of 640 x 480, D = 64, 1242 x 375, 128, 1280 x
+// 720, 192 and 1920 x 1080, 256: 38.5 ms with the best alone, 36.3 so)
+extern "C" sgmf_status sgmf_multi_autotune(sgmf_multi *m, int reps) {
+  if (!m) return mfail(SGMF_ERR_ARG, "sgmf_multi_autotune: NULL batch");
+  if (m->last) cudaStreamSynchronize(m->last);
+  drop_graph(m);
+  for (MultiClass &c : m->cls) {
+    sgmf_status st = sgmf_autotune(c.ctx, c.nf, c.left, c.right, c.lidar, c.out, reps, nullptr, nullptr);
+    if (st != SGMF_OK) return mfail(st, "sgmf_multi_autotune: %s", sgmf_last_error(c.ctx));
+  }
+  if (m->cls.size() < 2) return SGMF_OK;
+  float best = 0.0f;
+  sgmf_status st = time_batch(m, reps, &best);
+  for (size_t i = 0; i < m->cls.size() && st == SGMF_OK; ++i) {
+    sgmf_ctx *c = m->cls[i].ctx;
+    sgmf_tuning keep, other;
+    sgmf_get_tuning(c, &keep);
+    other = keep;
+    other.sweep = !keep.sweep;
+    other.line_warps = 4;                                  // (as the shapes alone were tried)
+    if (sgmf_set_tuning(c, &other) != SGMF_OK) continue;   // the sweep does not fit this class
+    float ms = 0.0f;
+    st = time_batch(m, reps, &ms);
+    if (st == SGMF_OK && ms < 0.99f * best)
+      best = ms;
+    else
+      sgmf_set_tuning(c, &keep);
+  }
+  return st;
 }
 
 extern "C" sgmf_status sgmf_multi_launch(sgmf_multi *m, void *stream) {
