@@ -15,10 +15,10 @@
 // minimum's four, a few words of bookkeeping) serves 4 Dp cells.  The 16-lane
 // groups of adjacent-cell words that this replaced spent two full-warp
 // reductions and Dp / 16 + 1 permutes per 2 Dp cells: at D = 128 a sweep over
-// six directions took 592 instructions per 512 cells, now 445 (1242 x 375, one
-// wave of frames: 786 -> 602 us).  A step and its minimum alone are 42
-// instructions at D = 128, 37 of them on the ALU pipe, 176 cycles from step to
-// step when nothing hides them and about 80 when two or more warps do.
+// six directions took 592 instructions per 512 cells, now 395 (1242 x 375, one
+// wave of frames: 786 -> 602 us).  A step of a line walk at D = 128, with its cost
+// bytes and its share of the stores, is 83 instructions for four vectors; where
+// few warps share a SM it takes about 146 ns (1242 steps in 181 us).
 //
 // A path start is the same step applied to an all-zero previous vector (with
 // m = 0 it yields L = C).  Disparities d >= D are padding: their cost is

@@ -93,8 +93,9 @@ struct WtaCfg {
 // one step of Eq. 2 from its predecessor, which lies in an even column (row)
 // and was stored; on the bands it is re-indexed first where it lies in another
 // tile.  Bytes come with neither or with both.  At D = 128 the kernel with byte
-// vectors then executes 565 instructions per 512 cells instead of 173 and is
-// ALU-bound: 8 frames of 1242 x 375 605 -> 760 us, the walks 1185 -> 857.  u16
+// vectors then executes 593 instructions per 512 cells instead of 351 and is
+// ALU-bound (79 % of the pipe): 8 frames of 1242 x 375 605 -> 760 us, the walks
+// 1185 -> 857.  u16
 // vectors come with RH at least: the rows' two directions then fit the region
 // that one sum of both took, whose second walk had to wait for the first and read
 // and write all of it (p2 = 300, 1242 x 375, D = 128: one frame 578 -> 439 us a call,
