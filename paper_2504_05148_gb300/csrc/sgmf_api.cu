@@ -588,14 +588,14 @@ static sgmf_status finish(sgmf_ctx *c, KParams ka, const Buffers &b, int nf, int
 // 1411 -> 1504 us, at Dp = 256 1920 x 1080 x 4 8550 -> 10460.
 // u16: the rows' vectors are half stored in any case (they share a region); the
 // other families' for 25 instead of 37 bytes a cell, earlier and at every width: 640 x
-// 480, D = 64 20 M cells 200 -> 228 us, 39 M 333 -> 336, 79 M 697 -> 565; 333 x 217,
-// D = 100 9 M 143 -> 150, 28 M 240 -> 216; 1920 x 1080 x 4, D = 256 12443 -> 10092.
-// Four paths: 28 M cells 162 -> 169, 60 M 317 -> 308, 123 M 551 -> 504.  Bands of
-// 64: 59 M 622 -> 654, 79 M 642 -> 620, 133 M 1208 -> 1222, 531 M 3969 -> 3756.
+// 480, D = 64 20 M cells 201 -> 227 us, 39 M 354 -> 340, 79 M 626 -> 576; 333 x 217,
+// D = 100 9 M 143 -> 150, 28 M 240 -> 218; 1920 x 1080 x 4, D = 256 12443 -> 10092.
+// Four paths: 39 M cells 221 -> 233, 60 M 317 -> 309, 123 M 551 -> 504.  Bands of
+// 64: 30 M 456 -> 482, 59 M 652 -> 670, 79 M 681 -> 629, 531 M 3969 -> 3756.
 static int half_vectors(const sgmf_ctx *c, int n) {
   const KParams &k = c->k;
   const size_t cells = frame_cells(k) * n;
-  if (!c->spill8) return cells >= (k.band ? 100000000u : (k.num_paths == 8 ? 25000000u : 50000000u));
+  if (!c->spill8) return cells >= (k.band ? 70000000u : (k.num_paths == 8 ? 25000000u : 50000000u));
   return !k.band && (k.Dp == 128 || k.Dp == 192) && cells >= (k.num_paths == 8 ? 100000000u : 200000000u);
 }
 

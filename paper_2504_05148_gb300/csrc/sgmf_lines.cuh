@@ -212,8 +212,19 @@ static cudaError_t launch_family(const LineArgs &a, int nf, bool overlap, cudaSt
   cfg.gridDim = dim3((lines + per_cta - 1) / per_cta, 2, nf);
   cfg.blockDim = dim3(32 * warps);
   cfg.dynamicSmemBytes = warps * kWarp;
+  // u16 at 8 cells a lane: one split of the L1 for every family.  An SM changes its
+  // split only when it is empty, and these families, left to the driver, asked for
+  // different ones: a family waited on every SM for those it overlaps (D = 64, four
+  // paths: the walks of 64 x 8192 2754 us, 692 so; of 12 frames of 160 x 90 69, 27).
+  // The others agree, and lose by a larger share of shared memory where they read
+  // through the L1: bands of 64 5 %, 24 cells a lane 10 %
   static bool done[64] = {};
-  const cudaError_t e = smem_optin(k_lines<CPL, S8, FAM, BANDED, HALF>, kMaxWarps * kWarp, done);
+  const cudaError_t e = once_per_device(done, [](int) {
+    auto kern = k_lines<CPL, S8, FAM, BANDED, HALF>;
+    const cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxWarps * kWarp);
+    if (r != cudaSuccess || S8 || BANDED || CPL > 8) return r;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  });
   if (e != cudaSuccess) return e;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -254,10 +265,7 @@ static cudaError_t launch_walks(const KParams &k, const Buffers &b, int nf, cuda
   a.gate = b.gate;
   a.lo = b.band_lo;
   // the first launch waits for the cost volume as usual; the others may start
-  // beside it (they touch nothing it writes).  The longest walks go first: those
-  // that start beside others' blocks land where these leave room, and few long
-  // ones then share a SM (64 x 8192, D = 64, u16, four paths: the walks 2757 us with
-  // the rows first, 688 so)
+  // beside it (they touch nothing it writes).  The rows, the longest walks, go first
   bool overlap = false;
   cudaError_t e = cudaSuccess;
   auto family = [&](auto fam) {
@@ -273,15 +281,13 @@ static cudaError_t launch_walks(const KParams &k, const Buffers &b, int nf, cuda
       e = launch_family<CPL, S8, F, BANDED, false>(a, nf, overlap, s);
     overlap = true;
   };
-  const bool tall = k.H > k.W && !k.rows_lines;
-  if (!tall) family(std::integral_constant<int, 3>{});
+  family(std::integral_constant<int, 3>{});
   if (k.rows_lines) return e;                       // the other directions are the sweep's
   family(std::integral_constant<int, 0>{});
   if (k.num_paths == 8) {
     family(std::integral_constant<int, 1>{});
     family(std::integral_constant<int, 2>{});
   }
-  if (tall) family(std::integral_constant<int, 3>{});
   return e;
 }
 
